@@ -240,24 +240,15 @@ void launch_ffwd(Ctx* c, const FwdArgs<T>& a, cudaStream_t s) {
   c->launches++;
 }
 
-template <class T>
-int launch_prec(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
-                bool virial = true) {
+// One translation unit per species count and path (fwd_f32.cu and the
+// fwd_f64*.cu files) instantiates this.
+template <class T, int NS>
+int launch_species(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s, bool virial) {
   FwdArgs<T> a = make_args<T>(c, f, acc, eatom, virial);
-  if (c->ablate & TERSOFF_ABLATE_FASTFWD) {
-    switch (c->ns) {
-      case 1: launch_ffwd<T, 1>(c, a, s); break;
-      case 2: launch_ffwd<T, 2>(c, a, s); break;
-      default: launch_ffwd<T, 0>(c, a, s); break;
-    }
-    TGB_CUDA(c, cudaGetLastError());
-    return TERSOFF_OK;
-  }
-  switch (c->ns) {
-    case 1: launch_buckets<T, 1>(c, a, s); break;
-    case 2: launch_buckets<T, 2>(c, a, s); break;
-    default: launch_buckets<T, 0>(c, a, s); break;
-  }
+  if (c->ablate & TERSOFF_ABLATE_FASTFWD)
+    launch_ffwd<T, NS>(c, a, s);
+  else
+    launch_buckets<T, NS>(c, a, s);
   TGB_CUDA(c, cudaGetLastError());
   return TERSOFF_OK;
 }

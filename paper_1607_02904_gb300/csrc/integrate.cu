@@ -54,7 +54,7 @@ __device__ __forceinline__ float pack_one(const PackArgs& a, int i, int t, doubl
                              (float)q2 * a.inv_scale, __int_as_float(t));
     a.qref[i] = make_int4(q0, q1, q2, t);
   }
-  if (a.fp64) a.pos64[i] = dpos4{x0 - o0, x1 - o1, x2 - o2, (double)t};
+  if (a.fp64) a.pos64[i] = dpos4{x0 - o0, x1 - o1, x2 - o2, __longlong_as_double((long long)t)};
   float d2 = 0.0f;
   if (a.track) {
     const float d0 = (float)(q0 - r.x) * a.inv_scale;

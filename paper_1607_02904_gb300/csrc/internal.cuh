@@ -13,7 +13,7 @@
 namespace tgb {
 
 // Position record of the FP64 path: offset from the atom's origin and its
-// species (as a double), 32-byte aligned for one wide load.
+// species (an integer in the low bits of w), 32-byte aligned for one wide load.
 struct alignas(32) dpos4 {
   double x, y, z, w;
 };
@@ -176,7 +176,7 @@ struct Ctx {
   unsigned long long* d_kmask = nullptr;  // n: short-list entries whose receiving slot may
                                           // hold a nonzero force (all ones after a build)
   int4* d_posq = nullptr;         // n: (u fixed point, type)
-  dpos4* d_pos64 = nullptr;     // n: (u double, type)
+  dpos4* d_pos64 = nullptr;     // n: (u double, type bits)
   int* d_flags = nullptr;         // device status words (see FLAG_*)
   int* h_flags = nullptr;         // pinned mirror
   double* d_acc = nullptr;        // ACC_LEN: energy, virial (6), kinetic at stride ACC_STRIDE
@@ -368,15 +368,17 @@ int launch_neighbor_export(Ctx* c, int* cnt, int* nbr, int cap, cudaStream_t s);
 // maximum displacement since the build is updated.
 int launch_pack_positions(Ctx* c, const double* x, bool build, cudaStream_t s);
 
-// Forces (fwd_f32.cu / fwd_f64.cu). Accumulates into f (zeroed by the caller),
+// Forces (fwd_f32.cu / fwd_f64*.cu). Accumulates into f (zeroed by the caller),
 // energy and virial into acc components 0..6 (zeroed by the caller); eatom optional.
 // virial false: acc receives the energy only (its virial components stay 0).
 int launch_forward(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
                    bool virial = true);
 int launch_forward_f32(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
                        bool virial);
-int launch_forward_f64(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
-                       bool virial);
+int launch_forward_f64_two(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
+                           bool virial);
+int launch_forward_f64_any(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
+                           bool virial);
 // the force launches of the TERSOFF_ABLATE_COMP_ATOM_SUMS variant (fwd_f32_cs.cu),
 // register capacity 4 or 8; args is a fwd::FwdArgs<float>
 int launch_forward_cs(Ctx* c, const void* args, int zc, int grid, cudaStream_t s);
@@ -388,6 +390,7 @@ int launch_forward_quad(Ctx* c, const void* args, bool ev, cudaStream_t s);
 // per-atom energy d_eatom and virial d_vatom.
 int launch_forward_batch(Ctx* c, double* f, cudaStream_t s);
 int launch_forward_batch_f32(Ctx* c, double* f, cudaStream_t s);
+int launch_forward_batch_f64(Ctx* c, double* f, cudaStream_t s);
 // Per-system sums of d_eatom and d_vatom: energy[n_sys], virial[n_sys x 6]
 // (either may be NULL).
 int launch_system_sums(Ctx* c, double* energy, double* virial, cudaStream_t s);

@@ -213,7 +213,7 @@ __global__ void k_bin_pack(int n, const double* __restrict__ x, const __grid_con
   bp.qref[i] = pq;
   bp.pos32[i] = make_float4((float)q3[0] * bp.inv_scale, (float)q3[1] * bp.inv_scale,
                             (float)q3[2] * bp.inv_scale, __int_as_float(t));
-  if (bp.pos64) bp.pos64[i] = dpos4{xr[0] - o3[0], xr[1] - o3[1], xr[2] - o3[2], (double)t};
+  if (bp.pos64) bp.pos64[i] = dpos4{xr[0] - o3[0], xr[1] - o3[1], xr[2] - o3[2], __longlong_as_double((long long)t)};
   bp.kmask[i] = ~0ull;
 }
 

@@ -65,19 +65,21 @@ template <> struct BM<float> {
     sincospif(x, s, c);
   }
   static __device__ __forceinline__ float sq(float x) { return sqrtf(x); }
+  static __device__ __forceinline__ float inv(float x) { return 1.0f / x; }
   // reciprocal: hardware approximation and one Newton step (~1 ulp)
   static __device__ __forceinline__ float rcp(float x) { return fwd::M<float>::rcp_nr(x); }
 };
 template <> struct BM<double> {
-  static __device__ __forceinline__ double ex(double x) { return exp(x); }
-  static __device__ __forceinline__ double ln(double x) { return log(x); }
+  static __device__ __forceinline__ double ex(double x) { return fx::exp(x); }
+  static __device__ __forceinline__ double ln(double x) { return fx::log(x); }
   static __device__ __forceinline__ double ln1p(double x) { return log1p(x); }
   static __device__ __forceinline__ double pw(double x, double y) { return pow(x, y); }
   static __device__ __forceinline__ void scpi(double x, double* s, double* c) {
-    sincospi(x, s, c);
+    fx::sincospi(x, s, c);
   }
-  static __device__ __forceinline__ double sq(double x) { return sqrt(x); }
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+  static __device__ __forceinline__ double sq(double x) { return x * fx::rsqrt(x); }
+  static __device__ __forceinline__ double rcp(double x) { return fx::rcp(x); }
+  static __device__ __forceinline__ double inv(double x) { return fx::rcp(x); }
 };
 
 // f_C(r; R, D), its r-derivative, and the R- and D-derivatives of both.
@@ -157,14 +159,16 @@ template <class T> struct Expo {
 template <class T>
 __device__ __forceinline__ Expo<T> expo_ad(T delta, T l3, int m) {
   Expo<T> o;
+  T mt;
+  fwd::small_real(m, mt);
   const T a = l3 * delta;
   T am1 = T(1);
   for (int s = 1; s < m; ++s) am1 *= a;
   const T am = am1 * a;
   o.x = am == T(0) ? T(1) : BM<T>::ex(am);  // lambda3 = 0 (most tables): no exponential
-  o.dx = T(m) * l3 * am1 * o.x;
-  o.x_l = T(m) * am1 * delta * o.x;
-  o.dx_l = T(m) * T(m) * am1 * (T(1) + am) * o.x;
+  o.dx = mt * l3 * am1 * o.x;
+  o.x_l = mt * am1 * delta * o.x;
+  o.dx_l = mt * mt * am1 * (T(1) + am) * o.x;
   return o;
 }
 
@@ -366,7 +370,7 @@ __device__ __forceinline__ void put_slot(T* sh, int q, const BondD<T>& b) {
   p[5 * B] = b.px;
   p[6 * B] = b.py;
   p[7 * B] = b.pz;
-  p[8 * B] = T(b.t);
+  fwd::put_int(p[8 * B], b.t);
 }
 template <class T>
 __device__ __forceinline__ void get_slot(const T* sh, int q, BondD<T>& b) {
@@ -380,7 +384,7 @@ __device__ __forceinline__ void get_slot(const T* sh, int q, BondD<T>& b) {
   b.px = p[5 * B];
   b.py = p[6 * B];
   b.pz = p[7 * B];
-  b.t = (int)p[8 * B];
+  b.t = fwd::get_int(p[8 * B]);
 }
 
 // The adjoint of L_i over the neighbourhood given by get(q, bond) for
@@ -416,7 +420,7 @@ __device__ __forceinline__ void atom_adjoint(const T* sraw, int ns, int ti, T hE
                                       rec_val(sraw, q, TERSOFF_P_D),
                                       rec_val(sraw, q, TERSOFF_P_H));
       const Expo<T> ex = expo_ad<T>(rj - rk, rec_val(sraw, q, TERSOFF_P_LAMBDA3),
-                                    (int)rec_val(sraw, q, TERSOFF_P_M));
+                                    fwd::small_int(rec_val(sraw, q, TERSOFF_P_M)));
       zeta += fk.fc * an.g * ex.x;
       zd += fk.dfc * rdk * an.g * ex.x + fk.fc * an.dg * csd * ex.x +
             fk.fc * an.g * ex.dx * (rdj - rdk);
@@ -472,7 +476,7 @@ __device__ __forceinline__ void atom_adjoint(const T* sraw, int ns, int ti, T hE
                                       rec_val(sraw, q, TERSOFF_P_H));
       const T dl = rj - rk, dld = rdj - rdk;
       const Expo<T> ex = expo_ad<T>(dl, rec_val(sraw, q, TERSOFF_P_LAMBDA3),
-                                    (int)rec_val(sraw, q, TERSOFF_P_M));
+                                    fwd::small_int(rec_val(sraw, q, TERSOFF_P_M)));
       // T = F3 G X ; T_rate = F3' rd_k G X + F3 G' cs_rate X + F3 G X' dl_rate
       const T F3bar = zbar * an.g * ex.x + zdbar * (an.dg * csd * ex.x + an.g * ex.dx * dld);
       const T F3dbar = zdbar * rdk * an.g * ex.x;
@@ -549,7 +553,7 @@ __global__ void __launch_bounds__(BwdBlock<T>::size) k_tersoff_bwd(const __grid_
       const T r2 = dx * dx + dy * dy + dz * dz;
       if (!(r2 <= sfilt[ti * ns + b.t])) return false;
       b.r = BM<T>::sq(r2);
-      const T ir = T(1) / b.r;
+      const T ir = BM<T>::inv(b.r);
       b.ux = dx * ir;
       b.uy = dy * ir;
       b.uz = dz * ir;
@@ -646,7 +650,7 @@ __device__ __forceinline__ D2<T> cutoff2(T r, T R, T D) {
 // g(cos) and its first two cos-derivatives (t = h - cos, Den = d^2 + t^2)
 template <class T>
 __device__ __forceinline__ D2<T> angular2(T cs, T ga, T c, T d, T h) {
-  const T t = h - cs, t2 = t * t, d2 = d * d, den = d2 + t2, iden = T(1) / den, c2 = c * c;
+  const T t = h - cs, t2 = t * t, d2 = d * d, den = d2 + t2, iden = BM<T>::inv(den), c2 = c * c;
   D2<T> o;
   o.f = ga + ga * c2 * t2 / (d2 * den);
   o.d1 = -T(2) * ga * c2 * t * iden * iden;
@@ -656,14 +660,16 @@ __device__ __forceinline__ D2<T> angular2(T cs, T ga, T c, T d, T h) {
 // X(Delta) = exp((lambda3 Delta)^m) and its first two Delta-derivatives
 template <class T>
 __device__ __forceinline__ D2<T> expo2(T delta, T l3, int m) {
+  T mt;
+  fwd::small_real(m, mt);
   const T a = l3 * delta;
   T am2 = T(1);  // a^(m-2), used for m >= 2
   for (int s = 2; s < m; ++s) am2 *= a;
   const T am1 = m >= 2 ? am2 * a : T(1);
   D2<T> o;
   o.f = BM<T>::ex(am1 * a);
-  o.d1 = T(m) * l3 * am1 * o.f;
-  o.d2 = (m >= 2 ? T(m) * T(m - 1) * l3 * l3 * am2 * o.f : T(0)) + T(m) * l3 * am1 * o.d1;
+  o.d1 = mt * l3 * am1 * o.f;
+  o.d2 = (m >= 2 ? mt * (mt - T(1)) * l3 * l3 * am2 * o.f : T(0)) + mt * l3 * am1 * o.d1;
   return o;
 }
 
@@ -682,7 +688,7 @@ __device__ __forceinline__ BondBar<T> zero_bar() {
 // r = |d|, u = d / r, rd = u . w, p = (w - u rd) / r (w held fixed).
 template <class T>
 __device__ __forceinline__ void bond_vec_bar(const BondD<T>& b, BondBar<T> q, T& dx, T& dy, T& dz) {
-  const T ir = T(1) / b.r;
+  const T ir = BM<T>::inv(b.r);
   q.ux -= b.rd * ir * q.px;
   q.uy -= b.rd * ir * q.py;
   q.uz -= b.rd * ir * q.pz;
@@ -708,7 +714,7 @@ template <class T, bool LAM3> struct Tri {
     G = angular2<T>(cs, rec_val(sraw, q, TERSOFF_P_GAMMA), rec_val(sraw, q, TERSOFF_P_C),
                     rec_val(sraw, q, TERSOFF_P_D), rec_val(sraw, q, TERSOFF_P_H));
     if constexpr (LAM3)
-      X = expo2<T>(rj - rk, rec_val(sraw, q, TERSOFF_P_LAMBDA3), (int)rec_val(sraw, q, TERSOFF_P_M));
+      X = expo2<T>(rj - rk, rec_val(sraw, q, TERSOFF_P_LAMBDA3), fwd::small_int(rec_val(sraw, q, TERSOFF_P_M)));
   }
 };
 
@@ -876,7 +882,7 @@ __global__ void __launch_bounds__(BS) k_tersoff_hvp(const __grid_constant__ BwdA
       const T r2 = dx * dx + dy * dy + dz * dz;
       if (!(r2 <= sfilt[ti * ns + bd.t])) return false;
       bd.r = BM<T>::sq(r2);
-      const T ir = T(1) / bd.r;
+      const T ir = BM<T>::inv(bd.r);
       bd.ux = dx * ir;
       bd.uy = dy * ir;
       bd.uz = dz * ir;

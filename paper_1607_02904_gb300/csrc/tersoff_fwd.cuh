@@ -27,6 +27,7 @@
 #pragma once
 #include <cstdint>
 
+#include "fxmath.cuh"
 #include "internal.cuh"
 
 namespace tgb {
@@ -71,6 +72,7 @@ template <> struct M<float> {
     float e = fmaf(-x, y, 1.0f);
     return fmaf(y, e, y);
   }
+  static __device__ __forceinline__ float inv(float x) { return 1.0f / x; }
   // exp(-(lh + ll) r) with the rounding residual of lh*r folded in
   static __device__ __forceinline__ float exp_neg_lr(float lh, float ll, float r) {
     float a = lh * r;
@@ -110,38 +112,55 @@ template <> struct M<float> {
   }
 };
 
+// Double path: reciprocals, exponentials and the bond order in 64-bit integer
+// arithmetic (fxmath.cuh), which leaves the FP64 pipe to the plain products
+// and sums.
 template <> struct M<double> {
-  static __device__ __forceinline__ double rsqrt_nr(double x) { return rsqrt(x); }
-  // reciprocal: the hardware approximation and two Newton steps on 1/y = x
-  // (each squares the relative error; the result is within about an ulp)
-  static __device__ __forceinline__ double rcp_nr(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    double e = fma(-x, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-x, y, 1.0);
-    return fma(y, e, y);
-  }
+  static __device__ __forceinline__ double rsqrt_nr(double x) { return fx::rsqrt(x); }
+  static __device__ __forceinline__ double rcp_nr(double x) { return fx::rcp(x); }
+  static __device__ __forceinline__ double inv(double x) { return fx::rcp(x); }
   static __device__ __forceinline__ double exp_neg_lr(double lh, double, double r) {
-    return exp(-lh * r);
+    return fx::exp(-lh * r);
   }
-  static __device__ __forceinline__ double exp_(double x) { return exp(x); }
+  static __device__ __forceinline__ double exp_(double x) { return fx::exp(x); }
   static __device__ __forceinline__ void sincospi_(double x, double* s, double* c) {
-    sincospi(x, s, c);
+    fx::sincospi(x, s, c);
+  }
+  // arguments outside the fixed-point formats
+  static __device__ __noinline__ void bond_wide(double zeta, double beta, double n, double ninv2,
+                                                double* b, double* db) {
+    double u = ::exp(n * ::log(beta * zeta));
+    *b = ::exp(ninv2 * log1p(u));
+    *db = -0.5 * *b * u / ((1.0 + u) * zeta);
   }
   static __device__ __forceinline__ void bond(double zeta, double beta, double n, double ninv2,
                                               double& b, double& db) {
     if (zeta > 0.0) {
-      double u = exp(n * log(beta * zeta));
-      double opu = 1.0 + u;
-      b = exp(ninv2 * log1p(u));
-      db = -0.5 * b * u * rcp_nr(opu * zeta);
+      if (!fx::bond(zeta, beta, n, ninv2, &b, &db)) bond_wide(zeta, beta, n, ninv2, &b, &db);
     } else {
       b = 1.0;
       db = 0.0;
     }
   }
 };
+
+// A small integer kept among values of type T as its bit pattern (conversions
+// between integers and doubles run on the FP64 pipe).
+__device__ __forceinline__ void put_int(float& w, int v) { w = __int_as_float(v); }
+__device__ __forceinline__ void put_int(double& w, int v) { w = __longlong_as_double((long long)v); }
+__device__ __forceinline__ int get_int(float w) { return __float_as_int(w); }
+__device__ __forceinline__ int get_int(double w) { return (int)__double_as_longlong(w); }
+// the integer value (1 to 16) of a table's m, and back
+__device__ __forceinline__ int small_int(float w) { return (int)w; }
+__device__ __forceinline__ int small_int(double w) {
+  const long long b = __double_as_longlong(w);
+  return (int)(((b & 0xfffffffffffffll) | 0x10000000000000ll) >> (1075 - (int)((b >> 52) & 0x7ff)));
+}
+__device__ __forceinline__ void small_real(int m, float& w) { w = (float)m; }
+__device__ __forceinline__ void small_real(int m, double& w) {
+  const int e = 31 - __clz(m);
+  w = m == 0 ? 0.0 : __hiloint2double(((1023 + e) << 20) | ((m << (20 - e)) & 0xfffff), 0);
+}
 
 // ---------------------------------------------------------------- arguments
 template <class T> struct FwdArgs {
@@ -214,7 +233,7 @@ template <> struct Pos<double> {
     x = p.x;
     y = p.y;
     z = p.z;
-    t = (int)p.w;
+    t = get_int(p.w);
   }
 };
 
@@ -224,6 +243,13 @@ __device__ __forceinline__ void decode(uint32_t e, int& j, int& ox, int& oy, int
   oy = (int)((e >> 28) & 3u) - 1;
   oz = (int)(e >> 30) - 1;
 }
+
+// o h for o in {-1, 0, 1}, by the bits of h
+__device__ __forceinline__ double times_unit(int o, double h) {
+  const long long b = __double_as_longlong(h) ^ ((long long)(o & 2) << 62);
+  return o == 0 ? 0.0 : __longlong_as_double(b);
+}
+__device__ __forceinline__ float times_unit(int o, float h) { return (float)o * h; }
 
 // Periodic shift units of atom i: the launch-wide cell edges, or (batches of
 // systems) those of atom i's system, loaded once per atom.
@@ -274,10 +300,10 @@ template <> struct Bond<double> {
     int ox, oy, oz;
     decode(e, j, ox, oy, oz);
     dpos4 pj = a.pos64[j];
-    dx = (pj.x - pi.x) + ox * sh.h(a, 0);
-    dy = (pj.y - pi.y) + oy * sh.h(a, 1);
-    dz = (pj.z - pi.z) + oz * sh.h(a, 2);
-    tj = (int)pj.w;
+    dx = (pj.x - pi.x) + times_unit(ox, sh.h(a, 0));
+    dy = (pj.y - pi.y) + times_unit(oy, sh.h(a, 1));
+    dz = (pj.z - pi.z) + times_unit(oz, sh.h(a, 2));
+    tj = get_int(pj.w);
   }
 };
 
@@ -370,12 +396,12 @@ __device__ __forceinline__ void triplet(const T* p3, T rij, T rik, T cs, T& zt, 
   T ex = T(1), dex = T(0);
   if (LAM3) {
     const T l3 = p3[K_LAM3];
-    const int m = (int)p3[K_M];
+    const int m = small_int(p3[K_M]);
     const T aa = l3 * (rij - rik);
     T am1 = T(1);
     for (int s = 1; s < m; ++s) am1 *= aa;
     ex = M<T>::exp_(am1 * aa);
-    dex = ex * T(m) * l3 * am1;
+    dex = ex * p3[K_M] * l3 * am1;
   }
   const T fg = fc * g;
   zt = fg * ex;
@@ -513,7 +539,7 @@ __device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T,
     const T rij = r2j * M<T>::rsqrt_nr(r2j);
     if (!(rij < p2[K_ROUT2])) continue;
     const T rexj = near_res(list[(size_t)sj * a.n + i], r2j, rij, tj);
-    const T rinj = T(1) / rij;
+    const T rinj = M<T>::inv(rij);
     const T uxj = dxj * rinj, uyj = dyj * rinj, uzj = dzj * rinj;
     T zeta = 0;
     for (int sk = 0; sk < c; ++sk) {
@@ -544,7 +570,7 @@ __device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T,
       const T r2k = dxk * dxk + dyk * dyk + dzk * dzk;
       const T rik = r2k * M<T>::rsqrt_nr(r2k);
       if (!(rik < p3[K_ROUT3])) continue;
-      const T rink = T(1) / rik;
+      const T rink = M<T>::inv(rik);
       const T uxk = dxk * rink, uyk = dyk * rink, uzk = dzk * rink;
       const T cs = uxj * uxk + uyj * uyk + uzj * uzk;
       T zt, A1, A2, A3;
@@ -889,9 +915,9 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
             T xj, yj, zj;
             int tj;
             Pos<T>::coarse(a, j, xj, yj, zj, tj);
-            const T dx = (xj - xi) + ox * sh.h(a, 0);
-            const T dy = (yj - yi) + oy * sh.h(a, 1);
-            const T dz = (zj - zi) + oz * sh.h(a, 2);
+            const T dx = (xj - xi) + times_unit(ox, sh.h(a, 0));
+            const T dy = (yj - yi) + times_unit(oy, sh.h(a, 1));
+            const T dz = (zj - zi) + times_unit(oz, sh.h(a, 2));
             const T r2 = dx * dx + dy * dy + dz * dz;
             if (r2 <= sfilt[ti * ns + tj]) mask |= 1ull << s;
           }
@@ -915,9 +941,9 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
           T xj, yj, zj;
           int tj;
           Pos<T>::coarse(a, j, xj, yj, zj, tj);
-          const T dx = (xj - xi) + ox * sh.h(a, 0);
-          const T dy = (yj - yi) + oy * sh.h(a, 1);
-          const T dz = (zj - zi) + oz * sh.h(a, 2);
+          const T dx = (xj - xi) + times_unit(ox, sh.h(a, 0));
+          const T dy = (yj - yi) + times_unit(oy, sh.h(a, 1));
+          const T dz = (zj - zi) + times_unit(oz, sh.h(a, 2));
           const T r2 = dx * dx + dy * dy + dz * dz;
           if (r2 <= sfilt[ti * ns + tj]) mask |= 1ull << s;
         }
@@ -1281,13 +1307,13 @@ __global__ void __launch_bounds__(WIDE_BLOCK) k_tersoff_wide(const __grid_consta
         if (!(r2 <= sfilt[ti * ns + tj])) continue;
         if (z < WIDE_SLOTS) {
           const T r = r2 * M<T>::rsqrt_nr(r2);
-          const T ir = T(1) / r;
+          const T ir = M<T>::inv(r);
           at(z, 0) = dx * ir;
           at(z, 1) = dy * ir;
           at(z, 2) = dz * ir;
           at(z, 3) = r;
-          at(z, 4) = T(tj);
-          at(z, 5) = T(s);
+          put_int(at(z, 4), tj);
+          put_int(at(z, 5), s);
           at(z, 6) = at(z, 7) = at(z, 8) = T(0);
           at(z, 9) = (sizeof(T) == 4 && r2 > snear[ti * ns + tj])
                          ? Exact<T>::residual(a, sh, pi, list[(size_t)s * a.n + i], r)
@@ -1308,14 +1334,14 @@ __global__ void __launch_bounds__(WIDE_BLOCK) k_tersoff_wide(const __grid_consta
     } else {
       for (int qj = 0; qj < z; ++qj) {
         const T uxj = at(qj, 0), uyj = at(qj, 1), uzj = at(qj, 2), rij = at(qj, 3);
-        const int tj = (int)at(qj, 4);
+        const int tj = get_int(at(qj, 4));
         const T* p2 = srec + rec_off<NS>(ns, ti, tj, tj);
         if (!(rij < p2[K_ROUT2])) continue;
         T zeta = 0;
         for (int qk = 0; qk < z; ++qk) {
           if (qk == qj) continue;
           const T rik = at(qk, 3);
-          const T* p3 = srec + rec_off<NS>(ns, ti, tj, (int)at(qk, 4));
+          const T* p3 = srec + rec_off<NS>(ns, ti, tj, get_int(at(qk, 4)));
           if (!(rik < p3[K_ROUT3])) continue;
           const T cs = uxj * at(qk, 0) + uyj * at(qk, 1) + uzj * at(qk, 2);
           T zt, A1, A2, A3;
@@ -1326,17 +1352,17 @@ __global__ void __launch_bounds__(WIDE_BLOCK) k_tersoff_wide(const __grid_consta
         pair<T>(p2, rij, zeta, V, dVdr, dzv, at(qj, 9));
         eatom_i += V;
         T Fjx = -dVdr * uxj, Fjy = -dVdr * uyj, Fjz = -dVdr * uzj;
-        const T rinj = T(1) / rij;
+        const T rinj = M<T>::inv(rij);
         for (int qk = 0; qk < z; ++qk) {
           if (qk == qj) continue;
           const T rik = at(qk, 3);
-          const T* p3 = srec + rec_off<NS>(ns, ti, tj, (int)at(qk, 4));
+          const T* p3 = srec + rec_off<NS>(ns, ti, tj, get_int(at(qk, 4)));
           if (!(rik < p3[K_ROUT3])) continue;
           const T uxk = at(qk, 0), uyk = at(qk, 1), uzk = at(qk, 2);
           const T cs = uxj * uxk + uyj * uyk + uzj * uzk;
           T zt, A1, A2, A3;
           triplet<T, LAM3>(p3, rij, rik, cs, zt, A1, A2, A3, at(qk, 9));
-          const T rink = T(1) / rik;
+          const T rink = M<T>::inv(rik);
           Fjx -= dzv * (A1 * (uxk - cs * uxj) * rinj + A2 * uxj);
           Fjy -= dzv * (A1 * (uyk - cs * uyj) * rinj + A2 * uyj);
           Fjz -= dzv * (A1 * (uzk - cs * uzj) * rinj + A2 * uzj);
@@ -1368,7 +1394,7 @@ __global__ void __launch_bounds__(WIDE_BLOCK) k_tersoff_wide(const __grid_consta
         w[3] += dx * fy;
         w[4] += dx * fz;
         w[5] += dy * fz;
-        const int s = (int)at(q, 5);
+        const int s = get_int(at(q, 5));
         if (slots) {
           store_slot<T>(a, a.contrib, recv_slot(a, s, i, entry_atom(a, list, s, i)), fx, fy, fz);
         } else {
@@ -1463,7 +1489,7 @@ __global__ void __launch_bounds__(BLOCK) k_tersoff_ffwd(const __grid_constant__ 
     while (__any_sync(FULL, sj < c)) {
       const bool act = sj < c;
       const T* p2 = srec + rec_off<NS>(ns, ti, tj, tj);
-      const T rinj = T(1) / rij;
+      const T rinj = M<T>::inv(rij);
       const T uxj = dxj * rinj, uyj = dyj * rinj, uzj = dzj * rinj;
       int sk = 0, k = i, tk = 0;
       T dxk = 0, dyk = 0, dzk = 0, rik = 1, rexk = 0;
@@ -1509,7 +1535,7 @@ __global__ void __launch_bounds__(BLOCK) k_tersoff_ffwd(const __grid_constant__ 
         if (!__any_sync(FULL, act && sk < c)) break;
         if (act && sk < c) {
           const T* p3 = srec + rec_off<NS>(ns, ti, tj, tk);
-          const T rink = T(1) / rik;
+          const T rink = M<T>::inv(rik);
           const T uxk = dxk * rink, uyk = dyk * rink, uzk = dzk * rink;
           const T cs = uxj * uxk + uyj * uyk + uzj * uzk;
           T zt, A1, A2, A3;
