@@ -115,7 +115,6 @@ int ensure_atoms(Ctx* c, int n) {
   int st;
   if ((st = dev_alloc(c, &c->d_types, m))) return st;
   if ((st = dev_alloc(c, &c->d_cnt, m))) return st;
-  if ((st = dev_alloc(c, &c->d_origin, 3 * m))) return st;
   if ((st = dev_alloc(c, &c->d_cell_of, m))) return st;
   if ((st = dev_alloc(c, &c->d_cell_atoms, m))) return st;
   if ((st = dev_alloc(c, &c->d_pos32, m))) return st;
@@ -197,6 +196,7 @@ int setup_grid(Ctx* c, const double* box, double r_list) {
   // offsets u = x - o stay within [-8, h + 8) A between rebuilds; 2^S such
   // that (h + 8) 2^S < 2^30 keeps differences inside int32
   g.fix_shift = (int)std::floor(30.0 - std::log2(hmax + 8.0));
+  g.fix64 = fix64_of(std::fmax(box[0], std::fmax(box[1], box[2])));
   return TERSOFF_OK;
 }
 
@@ -301,8 +301,8 @@ int tersoff_destroy(tersoff_ctx* p) {
   Ctx* c = &p->impl;
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
-  void* bufs[] = {c->d_rec64, c->d_rec32, c->d_raw64, c->d_raw32, c->d_filt64, c->d_filt32, c->d_near32,
-                  c->d_types, c->d_cnt, c->d_nbr, c->d_origin, c->d_cell_of, c->d_cell_count, c->d_cell_start,
+  void* bufs[] = {c->d_rec64, c->d_rec32, c->d_raw64, c->d_raw32, c->d_fx, c->d_filt32, c->d_near32,
+                  c->d_types, c->d_cnt, c->d_nbr, c->d_cell_of, c->d_cell_count, c->d_cell_start,
                   c->d_cell_fill, c->d_cell_atoms, c->d_scan_tmp, c->d_bintab, c->d_pos32, c->d_posc, c->d_kmask, c->d_zw, c->d_fine, c->d_zbins, c->d_posq,
                   c->d_pos64, c->d_flags, c->d_acc, c->d_fbuf, c->d_stage, c->d_thermo,
                   c->d_coef, c->d_qorg, c->d_qref, c->d_short, c->d_zcnt, c->d_trow,
@@ -434,17 +434,14 @@ int tersoff_params(tersoff_ctx* p, int ns, const double* table) {
       near32[(size_t)ti * ns + tx] = (float)(rl * rl);
       rmax = std::fmax(rmax, rf);
     }
-  std::vector<double> f64(filt.size());
   std::vector<float> f32(filt.size());
   for (size_t q = 0; q < filt.size(); ++q) {
     // a little above the radius so that rounding never drops a contributing atom
     double r = filt[q] * (1.0 + 1e-6);
-    f64[q] = r * r;
     f32[q] = (float)(r * r);
   }
   if ((st = tgb::dev_alloc(c, &c->d_rec64, r64.size()))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_rec32, r32.size()))) return st;
-  if ((st = tgb::dev_alloc(c, &c->d_filt64, f64.size()))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_filt32, f32.size()))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_near32, near32.size()))) return st;
   TGB_CUDA(c, cudaMemcpy(c->d_rec64, r64.data(), sizeof(double) * r64.size(), cudaMemcpyHostToDevice));
@@ -459,7 +456,6 @@ int tersoff_params(tersoff_ctx* p, int ns, const double* table) {
     TGB_CUDA(c, cudaMemcpy(c->d_raw64, table, sizeof(double) * nraw, cudaMemcpyHostToDevice));
     TGB_CUDA(c, cudaMemcpy(c->d_raw32, raw32.data(), sizeof(float) * nraw, cudaMemcpyHostToDevice));
   }
-  TGB_CUDA(c, cudaMemcpy(c->d_filt64, f64.data(), sizeof(double) * f64.size(), cudaMemcpyHostToDevice));
   TGB_CUDA(c, cudaMemcpy(c->d_filt32, f32.data(), sizeof(float) * f32.size(), cudaMemcpyHostToDevice));
   TGB_CUDA(c, cudaMemcpy(c->d_near32, near32.data(), sizeof(float) * near32.size(),
                          cudaMemcpyHostToDevice));
@@ -473,6 +469,11 @@ int tersoff_params(tersoff_ctx* p, int ns, const double* table) {
   c->sym_table = sym;
   c->rmax_cut = rmax;
   c->have_list = false;
+  tgb::make_fx_records(c);
+  if (c->fx_ok) {
+    if ((st = tgb::dev_alloc(c, &c->d_fx, c->h_fx.size()))) return st;
+    TGB_CUDA(c, cudaMemcpy(c->d_fx, c->h_fx.data(), sizeof(tgb::FxRec) * c->h_fx.size(), cudaMemcpyHostToDevice));
+  }
   return TERSOFF_OK;
 }
 
@@ -538,7 +539,7 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
   // one cell grid per system, cells numbered consecutively
   std::vector<tgb::GridDev> geo(n_sys);
   std::vector<tgb::SysShift> shifts(n_sys);
-  double hmax = 0.0;
+  double hmax = 0.0, lmax = 0.0;
   long cells = 0;
   for (int q = 0; q < n_sys; ++q) {
     tgb::GridDev& g = geo[q];
@@ -560,6 +561,7 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
       g.invh[a] = nc / L;
       g.hf[a] = (float)g.h[a];
       hmax = std::fmax(hmax, g.h[a]);
+      lmax = std::fmax(lmax, L);
       nq *= nc;
     }
     cells += nq;
@@ -574,13 +576,15 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
     G.invL[a] = G.invh[a] = 1.0 / hmax;
   }
   G.fix_shift = (int)std::floor(30.0 - std::log2(hmax + 8.0));
+  G.fix64 = tgb::fix64_of(lmax);
   const double scale = std::ldexp(1.0, G.fix_shift);
-  for (int q = 0; q < n_sys; ++q)
+  for (int q = 0; q < n_sys; ++q) {
     for (int a = 0; a < 3; ++a) {
       shifts[q].hq[a] = (int)std::llrint(geo[q].h[a] * scale);
       shifts[q].hf[a] = (float)geo[q].h[a];
-      shifts[q].h[a] = geo[q].h[a];
     }
+    shifts[q].box = tgb::make_box64(&boxes[3 * (size_t)q], G.fix64);
+  }
   std::vector<int> asys((size_t)n);
   for (int q = 0; q < n_sys; ++q)
     for (int i = sys_offsets[q]; i < sys_offsets[q + 1]; ++i) asys[i] = q;

@@ -1,6 +1,8 @@
 // Host-side instantiation and launch of the force kernel for one precision.
 #pragma once
-#include "tersoff_fwd.cuh"
+#include <algorithm>
+
+#include "tersoff_lanes64.cuh"
 
 namespace tgb {
 namespace fwd {
@@ -11,9 +13,6 @@ template <> inline const double* rec_ptr<double>(Ctx* c) { return c->d_rec64; }
 template <class T> const T* rec_host(Ctx* c);
 template <> inline const float* rec_host<float>(Ctx* c) { return c->h_rec32.data(); }
 template <> inline const double* rec_host<double>(Ctx* c) { return c->h_rec64.data(); }
-template <class T> const T* filt_ptr(Ctx* c);
-template <> inline const float* filt_ptr<float>(Ctx* c) { return c->d_filt32; }
-template <> inline const double* filt_ptr<double>(Ctx* c) { return c->d_filt64; }
 
 // Atoms with more than 8 bonds inside the cutoffs (bucket 2), when they are
 // over 0.5% of the atoms (e.g. SiC): the slot-cached wide kernel, on the
@@ -46,6 +45,17 @@ int ev_mode(const FwdArgs<T>& a) {
   return a.eatom != nullptr ? 1 : 0;
 }
 
+// MODE by the table: 1 with a lambda3 term, 2 symmetric without one, else 0.
+template <class T, int NS, int ZC, bool BATCH, int EV>
+void launch_mode(Ctx* c, const FwdArgs<T>& a, int grid, cudaStream_t s) {
+  if (c->has_lam3)
+    launch_pdl(k_tersoff<T, NS, ZC, 1, BATCH, false, EV>, grid, BLOCK, 0, s, a);
+  else if (c->sym_table)
+    launch_pdl(k_tersoff<T, NS, ZC, 2, BATCH, false, EV>, grid, BLOCK, 0, s, a);
+  else
+    launch_pdl(k_tersoff<T, NS, ZC, 0, BATCH, false, EV>, grid, BLOCK, 0, s, a);
+}
+
 // Grids are fixed by the atom count (the bucket sizes live on the device), so
 // the launches can be captured in a CUDA graph and replayed across builds.
 template <class T, int NS, int ZC, bool BATCH = false>
@@ -58,27 +68,19 @@ void launch_t(Ctx* c, const FwdArgs<T>& a, int grid, cudaStream_t s) {
   // forces only, or energy without the virial (MD steps, with or without
   // thermo): the instances with less bookkeeping
   const int evm = ev_mode<T, BATCH>(a);
-  if (ZC == 4 && !BATCH && evm == 0) {
-    if (c->has_lam3)
-      launch_pdl(k_tersoff<T, NS, ZC, 1, false, false, 0>, grid, BLOCK, 0, s, a);
-    else if (c->sym_table)
-      launch_pdl(k_tersoff<T, NS, ZC, 2, false, false, 0>, grid, BLOCK, 0, s, a);
-    else
-      launch_pdl(k_tersoff<T, NS, ZC, 0, false, false, 0>, grid, BLOCK, 0, s, a);
-  } else if (ZC == 4 && !BATCH && evm == 1) {
-    if (c->has_lam3)
-      launch_pdl(k_tersoff<T, NS, ZC, 1, false, false, 1>, grid, BLOCK, 0, s, a);
-    else if (c->sym_table)
-      launch_pdl(k_tersoff<T, NS, ZC, 2, false, false, 1>, grid, BLOCK, 0, s, a);
-    else
-      launch_pdl(k_tersoff<T, NS, ZC, 0, false, false, 1>, grid, BLOCK, 0, s, a);
-  } else if (c->has_lam3) {
-    launch_pdl(k_tersoff<T, NS, ZC, 1, BATCH>, grid, BLOCK, 0, s, a);
-  } else if (c->sym_table) {
-    launch_pdl(k_tersoff<T, NS, ZC, 2, BATCH>, grid, BLOCK, 0, s, a);
-  } else {
-    launch_pdl(k_tersoff<T, NS, ZC, 0, BATCH>, grid, BLOCK, 0, s, a);
+  if constexpr (ZC == 4 && !BATCH) {
+    if (evm == 0) {
+      launch_mode<T, NS, ZC, BATCH, 0>(c, a, grid, s);
+      c->launches++;
+      return;
+    }
+    if (evm == 1) {
+      launch_mode<T, NS, ZC, BATCH, 1>(c, a, grid, s);
+      c->launches++;
+      return;
+    }
   }
+  launch_mode<T, NS, ZC, BATCH, 2>(c, a, grid, s);
   c->launches++;
 }
 
@@ -114,8 +116,41 @@ bool use_quad(const Ctx* c) {
   return c->opt_quad == 1;
 }
 
+// The FP64 path's terms run one lane per bond (tersoff_lanes64.cuh) for tables
+// inside the integer formats; other tables, and the ablation that sends every
+// atom through Algorithm 2's loops, keep k_tersoff.
+inline bool use_lanes64(const Ctx* c) { return c->fx_ok && !(c->ablate & TERSOFF_ABLATE_GENERAL); }
+
+template <int NS, int W, bool BATCH, int EV>
+void launch_lanes_ev(Ctx* c, const FwdArgs<double>& a, int grid, cudaStream_t s) {
+  const bool sym = c->sym_table;  // (false with a lambda3 term)
+  void (*k)(FwdArgs<double>) = sym ? k_lanes64<NS, W, 3, BATCH, EV> : k_lanes64<NS, W, 1, BATCH, EV>;
+  const size_t dyn = lanes_dyn(sym ? 3 : 1);
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+  launch_pdl(k, grid, LBLOCK, dyn, s, a);
+  c->launches++;
+}
+// items: about how many atoms the launch has (the device's counts decide; the
+// kernel loops over what its grid does not cover)
+template <int NS, int W, bool BATCH>
+void launch_lanes(Ctx* c, const FwdArgs<double>& a, long long items, cudaStream_t s) {
+  constexpr int ATOMS = LBLOCK / W;
+  const long long full = ((long long)c->n + ATOMS - 1) / ATOMS;
+  long long grid = (items + ATOMS - 1) / ATOMS + (items < c->n ? 8 : 0);
+  if (c->opt_waves > 0 && c->n_sm > 0) grid = std::min(grid, (long long)c->opt_waves * c->n_sm * 5);
+  grid = std::max(1ll, std::min(grid, full));
+  const int evm = ev_mode<double, BATCH>(a);
+  if constexpr (W == 4 && !BATCH) {
+    if (evm == 0) return launch_lanes_ev<NS, W, BATCH, 0>(c, a, (int)grid, s);
+    if (evm == 1) return launch_lanes_ev<NS, W, BATCH, 1>(c, a, (int)grid, s);
+  }
+  launch_lanes_ev<NS, W, BATCH, 2>(c, a, (int)grid, s);
+}
+
 template <class T, int NS, bool BATCH = false>
 void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
+  constexpr bool D = sizeof(T) == 8;
+  const bool lanes = D && use_lanes64(c);
   if (use_quad<T, NS, BATCH>(c)) {
     TimedRegion tr(c, 0, s);
     const bool ev = a.acc != nullptr || a.eatom != nullptr;
@@ -151,7 +186,10 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
     b1.order2 = b1.order3 = nullptr;
     b1.n_items2 = b1.n_items3 = nullptr;
     b1.identity = 0;
-    launch_t<T, NS, 8, BATCH>(c, b1, force_grid(c, 8, ev_mode<T, BATCH>(a)), s2);
+    if constexpr (D) {
+      if (lanes) launch_lanes<NS, 8, BATCH>(c, b1, c->nbucket[1], s2);
+    }
+    if (!lanes) launch_t<T, NS, 8, BATCH>(c, b1, force_grid(c, 8, ev_mode<T, BATCH>(a)), s2);
   }
   // bucket 0, then bucket 1 (unless split off), then bucket 2 (general path)
   const bool wide = (dec & 2) != 0;
@@ -167,8 +205,25 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
   b0.identity = (split1 || wide) ? 0 : 1;
   {
     TimedRegion tr(c, 0, s);
-    launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
-    if (wide) launch_wide<T, NS, BATCH>(c, a, s);
+    if constexpr (D) {
+      if (lanes) {
+        long long items = c->n;
+        if (split1) items -= c->nbucket[1];
+        if (wide) items -= c->nbucket[2];
+        launch_lanes<NS, 4, BATCH>(c, b0, items, s);
+        if (wide) {
+          FwdArgs<T> b2 = a;
+          b2.order = c->d_bucket + 2 * (size_t)c->n;
+          b2.n_items = c->d_flags + flag_bucket(2);
+          b2.identity = 0;
+          launch_lanes<NS, 16, BATCH>(c, b2, c->nbucket[2], s);
+        }
+      }
+    }
+    if (!lanes) {
+      launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
+      if (wide) launch_wide<T, NS, BATCH>(c, a, s);
+    }
   }
   if (fork) {
     cudaEventRecord(c->ev_join, c->side);
@@ -187,14 +242,20 @@ FwdArgs<T> make_args(Ctx* c, double* f, double* acc, double* eatom, bool virial 
   a.cnt = c->d_cnt;
   a.pos32 = c->d_pos32;
   a.posq = c->d_posq;
-  a.pos64 = c->d_pos64;
   a.rec = rec_ptr<T>(c);
   for (int q = 0; q < RSTRIDE; ++q) a.prm1[q] = rec_host<T>(c)[q];
-  a.filt2 = filt_ptr<T>(c);
+  a.filt2 = c->d_filt32;
+  set_pos64(c, a);
+  if constexpr (sizeof(T) == 8) {
+    if (c->fx_ok) a.fx1 = c->h_fx[0];
+    a.fx = c->d_fx;
+    a.qd = c->fx_qd;
+    a.cut_j = c->fx_cut_j ? 1 : 0;
+  }
   a.near2 = c->d_near32;
   const double scale = ldexp(1.0, c->grid.fix_shift);
   for (int q = 0; q < 3; ++q) {
-    a.h[q] = (T)c->grid.h[q];
+    a.h[q] = (float)c->grid.h[q];
     a.hq[q] = (int)llrint(c->grid.h[q] * scale);
   }
   a.qinv = ldexpf(1.0f, -c->grid.fix_shift);

@@ -2,6 +2,7 @@
 // velocity-Verlet kick/drift on the FP64 state (x, v, f).
 #include "gather.cuh"
 #include "internal.cuh"
+#include "pos64.cuh"
 
 namespace tgb {
 namespace {
@@ -12,37 +13,36 @@ constexpr double ROUND_MAGIC = 6755399441055744.0;
 
 struct PackArgs {
   int n;
-  const double* origin;  // o_i (FP64 path offsets)
   const double* qorg;    // 1.5*2^52 - o_i 2^S
   int4* qref;            // offsets at the build (displacement tracking)
   const int* types;
-  int fp64;              // also write FP64 offsets
+  int fp64;              // also write the FP64 path's positions
   int track;             // update the running max displacement
   int build;             // at a build: float offsets and displacement references
   double scale;          // 2^S
   float inv_scale;       // 2^-S
   float4* pos32;
   int4* posq;
-  dpos4* pos64;
+  ipos4* pos64;
+  int fix64;
+  Box64 box;             // of a single system ...
+  const SysShift* sys;   // ... or the systems' (batches) and each atom's system
+  const int* atom_sys;
   int* flags;
 };
 
 // Packs atom i (species t) at position (x0, x1, x2); qo: its fixed-point
 // origin words; returns its squared displacement since the build (A^2) when
 // tracking. Loads are issued before any store.
+// P64: the FP64 path's positions may be wanted (instances of the mixed path
+// leave their arithmetic out, which costs registers).
+template <bool P64>
 __device__ __forceinline__ float pack_one(const PackArgs& a, int i, int t, double x0, double x1,
                                           double x2) {
   const double* qo = a.qorg + 3 * (size_t)i;
   const double qo0 = qo[0], qo1 = qo[1], qo2 = qo[2];
   int4 r = make_int4(0, 0, 0, 0);
   if (a.track) r = a.qref[i];
-  double o0 = 0.0, o1 = 0.0, o2 = 0.0;
-  if (a.fp64) {
-    const double* o = a.origin + 3 * (size_t)i;
-    o0 = o[0];
-    o1 = o[1];
-    o2 = o[2];
-  }
   // q = round((x - o) 2^S) with one rounding: fma(x, 2^S, magic - o 2^S)
   const long long mb = __double_as_longlong(ROUND_MAGIC);
   const int q0 = (int)(__double_as_longlong(fma(x0, a.scale, qo0)) - mb);
@@ -54,7 +54,12 @@ __device__ __forceinline__ float pack_one(const PackArgs& a, int i, int t, doubl
                              (float)q2 * a.inv_scale, __int_as_float(t));
     a.qref[i] = make_int4(q0, q1, q2, t);
   }
-  if (a.fp64) a.pos64[i] = dpos4{x0 - o0, x1 - o1, x2 - o2, __longlong_as_double((long long)t)};
+  if (P64 && a.fp64) {
+    if (a.sys)
+      a.pos64[i] = make_pos64(x0, x1, x2, t, a.fix64, a.sys[a.atom_sys[i]].box);
+    else
+      a.pos64[i] = make_pos64(x0, x1, x2, t, a.fix64, a.box);
+  }
   float d2 = 0.0f;
   if (a.track) {
     const float d0 = (float)(q0 - r.x) * a.inv_scale;
@@ -79,13 +84,14 @@ __device__ __forceinline__ void track_max(const PackArgs& a, float d2) {
   }
 }
 
-__global__ void k_pack(PackArgs a, const double* __restrict__ x) {
+template <bool P64>
+__global__ void k_pack(const __grid_constant__ PackArgs a, const double* __restrict__ x) {
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float d2 = 0.0f;
   if (i < a.n) {
     const double* xi = x + 3 * (size_t)i;
-    d2 = pack_one(a, i, a.types[i], xi[0], xi[1], xi[2]);
+    d2 = pack_one<P64>(a, i, a.types[i], xi[0], xi[1], xi[2]);
   }
   track_max(a, d2);
 }
@@ -150,7 +156,7 @@ __device__ __forceinline__ void block_sum_add(double v, double* dst) {
 // snap (first step of a call, MG false; may be null): receives x, v and f as
 // read (three n x 3 blocks), the state a rerun of the call starts from.
 template <bool MG, bool KE>
-__global__ void k_step(PackArgs pk, GatherArgs ga, int gather_, double* __restrict__ x,
+__global__ void k_step(const __grid_constant__ PackArgs pk, const __grid_constant__ GatherArgs ga, int gather_, double* __restrict__ x,
                        double* __restrict__ v, const double* __restrict__ f, const __grid_constant__ Coef cf,
                        double dt, int kick, int do_pack, double* ke_row_, double* acc_zero,
                        double* __restrict__ snap) {
@@ -241,7 +247,7 @@ __global__ void k_step(PackArgs pk, GatherArgs ga, int gather_, double* __restri
     x[b] = xn0;
     x[b + 1] = xn1;
     x[b + 2] = xn2;
-    if (do_pack) d2 = pack_one(pk, i, t, xn0, xn1, xn2);
+    if (do_pack) d2 = pack_one<!MG>(pk, i, t, xn0, xn1, xn2);
   }
   if (do_pack) track_max(pk, d2);
   if (ke_row) {
@@ -386,7 +392,6 @@ __global__ void k_thermo_rows(const double* rows, int nsteps, double mvv2e, doub
 PackArgs make_pack(Ctx* c, bool track, bool build = false) {
   PackArgs a;
   a.n = c->n;
-  a.origin = c->d_origin;
   a.qorg = c->d_qorg;
   a.qref = c->d_qref;
   a.types = c->d_types;
@@ -398,6 +403,10 @@ PackArgs make_pack(Ctx* c, bool track, bool build = false) {
   a.pos32 = c->d_pos32;
   a.posq = c->d_posq;
   a.pos64 = c->d_pos64;
+  a.fix64 = c->grid.fix64;
+  a.box = make_box64(c->grid.L, c->grid.fix64);
+  a.sys = c->n_sys > 0 ? c->d_sys : nullptr;
+  a.atom_sys = c->d_atom_sys;
   a.flags = c->d_flags;
   return a;
 }
@@ -407,7 +416,8 @@ PackArgs make_pack(Ctx* c, bool track, bool build = false) {
 int launch_pack_positions(Ctx* c, const double* x, bool build, cudaStream_t s) {
   if (c->n == 0) return TERSOFF_OK;
   const int B = c->opt_block;
-  TGB_CUDA(c, launch_pdl(k_pack, (c->n + B - 1) / B, B, 0, s, make_pack(c, !build, build), x));
+  TGB_CUDA(c, launch_pdl(c->precision == TERSOFF_FP64 ? k_pack<true> : k_pack<false>, (c->n + B - 1) / B, B, 0, s,
+                         make_pack(c, !build, build), x));
   c->launches++;
   TGB_CUDA(c, cudaGetLastError());
   return TERSOFF_OK;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -12,10 +13,19 @@
 
 namespace tgb {
 
-// Position record of the FP64 path: offset from the atom's origin and its
-// species (an integer in the low bits of w), 32-byte aligned for one wide load.
+// Force record of the FP64 path, 32-byte aligned for one wide store.
 struct alignas(32) dpos4 {
   double x, y, z, w;
+};
+
+// Position record of the FP64 path: the coordinates wrapped into the box, in
+// 64-bit fixed point with Grid::fix64 fraction bits (finer than a double's at
+// any coordinate from the middle of the box up, at most 2^-53 A off below),
+// and the species. Differences are exact integers, and a box edge (rounded
+// once) is added or subtracted where the minimum image asks for it: bond
+// vectors carry none of the rounding of cell origins.
+struct alignas(32) ipos4 {
+  long long x, y, z, w;
 };
 
 // ------------------------------------------------------------------ parameters
@@ -54,6 +64,19 @@ enum : int {
   RSTRIDE = 32
 };
 
+// Record of the FP64 path's integer arithmetic (tersoff_fx.cuh): mantissas
+// (64 bits, top bit set) with exponents _e, and fixed-point values.
+struct FxRec {
+  double gamma, hl1, hl2;   // gamma, lambda1/2, lambda2/2
+  long long h;              // 60 fraction bits
+  unsigned long long d2;    // d^2 with 64 - qden fraction bits
+  unsigned long long gc2d2, g2c2;  // gamma c^2/d^2, 2 gamma c^2
+  unsigned long long l1, l2;       // lambda1 log2(e), lambda2 log2(e)
+  unsigned long long n, in2;       // n, 1/(2n)
+  long long lgA, lgB, lgbeta;      // log2, 57 fraction bits
+  int qden, gc2d2_e, g2c2_e, l1_e, l2_e, n_e, in2_e, pad;
+};
+
 // ------------------------------------------------------------------ neighbour entries
 // Entry = j | (ox+1) << 26 | (oy+1) << 28 | (oz+1) << 30 where (ox,oy,oz) in
 // {-1,0,1}^3 is the cell offset of the image of j found from i's cell.
@@ -68,6 +91,7 @@ struct Grid {
   double h[3];    // cell edge L / nc
   double invh[3]; // nc / L
   int fix_shift;  // fixed-point scale 2^fix_shift for mixed positions
+  int fix64;      // scale 2^fix64 of the FP64 path's positions
 };
 
 // MD coefficients per species: c = dt/2 * (force-to-acceleration) / m, and m
@@ -89,13 +113,34 @@ struct GridDev {
   float hf[3];
 };
 
+// Box edges for the FP64 path: in fixed point (scale 2^fix64), and 1 / L.
+struct Box64 {
+  long long L[3];
+  double invL[3];
+  float invLf[3];
+};
+inline Box64 make_box64(const double* L, int fix64) {
+  Box64 b;
+  for (int a = 0; a < 3; ++a) {
+    b.L[a] = llrint(ldexp(L[a], fix64));
+    b.invL[a] = 1.0 / L[a];
+    b.invLf[a] = (float)b.invL[a];
+  }
+  return b;
+}
+// A scale that leaves int64 room for differences over two boxes.
+inline int fix64_of(double lmax) {
+  const int e = (int)ceil(log2(lmax));
+  return e <= 8 ? 52 : 60 - e;
+}
+
 // Periodic shift units of one system of a batch: the edges of its list cells,
-// in fixed point (mixed path), float and double. A list entry's cell offset
+// in fixed point and float (mixed path), and its box (FP64 path). A list entry's cell offset
 // code multiplies these.
 struct SysShift {
   int hq[3];
   float hf[3];
-  double h[3];
+  Box64 box;
 };
 
 // ------------------------------------------------------------------ context
@@ -112,14 +157,18 @@ struct Ctx {
   float* d_rec32 = nullptr;
   double* d_raw64 = nullptr;      // raw table (backward pass), device
   float* d_raw32 = nullptr;
+  FxRec* d_fx = nullptr;          // integer records (valid when fx_ok)
+  std::vector<FxRec> h_fx;
+  bool fx_ok = false;             // the table is inside the integer formats
+  int fx_qd = 0;                  // fraction bits of its bond vectors
+  bool fx_cut_j = false;          // f_C(r_ik) does not depend on j
   std::vector<double> h_rec64;    // host copies
   std::vector<float> h_rec32;
   cudaStream_t side = nullptr;    // side stream for small force launches
   cudaStream_t cap_stream = nullptr;  // stream used to capture MD graphs
   cudaStream_t body_stream = nullptr; // captures the body of a conditional rebuild
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-  double* d_filt64 = nullptr;     // (ti,tj) filter radius^2
-  float* d_filt32 = nullptr;
+  float* d_filt32 = nullptr;      // (ti,tj) filter radius^2
   float* d_near32 = nullptr;      // (ti,tj): squared (smallest outer cutoff - 2e-3 A); bonds
                                   // beyond it get their exact length residual (float path)
   std::vector<double> filt;       // host copy, radius (not squared)
@@ -138,7 +187,6 @@ struct Ctx {
   int* d_types = nullptr;         // n
   int* d_cnt = nullptr;           // n
   uint32_t* d_nbr = nullptr;      // cap * n, slot-major: nbr[s * n + i]
-  double* d_origin = nullptr;     // n x 3: o_i, u_i = x_i - o_i
   int* d_cell_of = nullptr;       // n
   int* d_cell_count = nullptr;    // ncell + 1
   int* d_cell_start = nullptr;    // ncell + 1
@@ -176,7 +224,7 @@ struct Ctx {
   unsigned long long* d_kmask = nullptr;  // n: short-list entries whose receiving slot may
                                           // hold a nonzero force (all ones after a build)
   int4* d_posq = nullptr;         // n: (u fixed point, type)
-  dpos4* d_pos64 = nullptr;     // n: (u double, type bits)
+  ipos4* d_pos64 = nullptr;       // n: FP64 path's positions
   int* d_flags = nullptr;         // device status words (see FLAG_*)
   int* h_flags = nullptr;         // pinned mirror
   double* d_acc = nullptr;        // ACC_LEN: energy, virial (6), kinetic at stride ACC_STRIDE
@@ -344,6 +392,9 @@ inline bool comp_atom_sums(const Ctx* c) {
          c->ns == 1 && c->n_sys == 0;
 }
 
+// The integer records of a table (params_fx.cu): c->fx_ok, h_fx, fx_qd.
+void make_fx_records(Ctx* c);
+
 int fail(Ctx* c, int code, const std::string& msg);
 int cuda_fail(Ctx* c, cudaError_t e, const char* where);
 
@@ -354,7 +405,7 @@ int cuda_fail(Ctx* c, cudaError_t e, const char* where);
   } while (0)
 
 // ------------------------------------------------------------------ launchers
-// Neighbour build (neighbor.cu). Fills d_nbr, d_cnt, d_origin; does not sync.
+// Neighbour build (neighbor.cu). Fills d_nbr, d_cnt; does not sync.
 int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s);
 // Per-axis binning tables of the single-system grid c->grid (cell thresholds,
 // origins and fixed-point origins), uploaded on s; called whenever that grid

@@ -1,7 +1,7 @@
 // Cell-binned full neighbour lists (Sec. II Eq. 4; skin of Sec. III).
 //
 // Pipeline, all on the caller's stream:
-//   k_bin      atom -> cell (wrapped position), per-atom origin o_i, FP32 offset
+//   k_bin      atom -> cell (wrapped position), fixed-point origin, FP32 offset
 //   scan       exclusive prefix sum of cell counts (three kernels)
 //   k_scatter  atoms grouped by cell
 //   k_neigh    one thread per atom scans the 27 stencil cells; candidates far from
@@ -15,6 +15,7 @@
 #include <cstring>
 
 #include "internal.cuh"
+#include "pos64.cuh"
 
 namespace tgb {
 namespace {
@@ -54,8 +55,7 @@ template <bool BATCH>
 __global__ void k_bin(int n, const double* __restrict__ x, const __grid_constant__ GridDev g1,
                       const GridDev* __restrict__ geo, const int* __restrict__ atom_sys,
                       double scale, int* __restrict__ cell_of, int* __restrict__ cell_count,
-                      double* __restrict__ origin, double* __restrict__ qorg,
-                      int* __restrict__ flags) {
+                      double* __restrict__ qorg, int* __restrict__ flags) {
   pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -87,7 +87,6 @@ __global__ void k_bin(int n, const double* __restrict__ x, const __grid_constant
       c = c < 0 ? 0 : (c >= g.nc[a] ? g.nc[a] - 1 : c);
       o = fma(k, g.L[a], c * g.h[a]);
     }
-    origin[3 * (size_t)i + a] = o;
     qorg[3 * (size_t)i + a] = 6755399441055744.0 - o * scale;
     c3[a] = c;
   }
@@ -124,14 +123,18 @@ struct BinPack {
   int4* posq;
   float4* pos32;
   int4* qref;
-  dpos4* pos64;  // FP64 path only, else null
+  ipos4* pos64;
+  int fix64;
+  Box64 box;
   unsigned long long* kmask;  // set to all ones (every slot may hold a stale force)
 };
 
+// P64: the FP64 path's positions are written too
+template <bool P64>
 __global__ void k_bin_pack(int n, const double* __restrict__ x, const __grid_constant__ GridDev g,
                            const __grid_constant__ BinPack bp, int* __restrict__ cell_of,
-                           int* __restrict__ cell_count, double* __restrict__ origin,
-                           double* __restrict__ qorg, int* __restrict__ flags) {
+                           int* __restrict__ cell_count, double* __restrict__ qorg,
+                           int* __restrict__ flags) {
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -199,7 +202,6 @@ __global__ void k_bin_pack(int n, const double* __restrict__ x, const __grid_con
       qo3[a] = 6755399441055744.0 - o3[a] * bp.scale;
     }
     c3[a] = c;
-    origin[3 * (size_t)i + a] = o3[a];
     qorg[3 * (size_t)i + a] = qo3[a];
     // the pack of k_pack at a build: q = round((x - o) 2^S) with one rounding
     q3[a] = (int)(__double_as_longlong(fma(xr[a], bp.scale, qo3[a])) - mb);
@@ -213,7 +215,7 @@ __global__ void k_bin_pack(int n, const double* __restrict__ x, const __grid_con
   bp.qref[i] = pq;
   bp.pos32[i] = make_float4((float)q3[0] * bp.inv_scale, (float)q3[1] * bp.inv_scale,
                             (float)q3[2] * bp.inv_scale, __int_as_float(t));
-  if (bp.pos64) bp.pos64[i] = dpos4{xr[0] - o3[0], xr[1] - o3[1], xr[2] - o3[2], __longlong_as_double((long long)t)};
+  if (P64) bp.pos64[i] = make_pos64(xr[0], xr[1], xr[2], t, bp.fix64, bp.box);
   bp.kmask[i] = ~0ull;
 }
 
@@ -703,7 +705,7 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
     if (batch) {
       // per-system grids: k_bin's arithmetic, then the build's pack
       TGB_CUDA(c, launch_pdl(k_bin<true>, nb, B, 0, s, n, x, g, c->d_geo, c->d_atom_sys, scale,
-                             c->d_cell_of, c->d_cell_count, c->d_origin, c->d_qorg, c->d_flags));
+                             c->d_cell_of, c->d_cell_count, c->d_qorg, c->d_flags));
       int st = launch_pack_positions(c, x, true, s);
       if (st) return st;
     } else {
@@ -716,10 +718,12 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
       bp.posq = c->d_posq;
       bp.pos32 = c->d_pos32;
       bp.qref = c->d_qref;
-      bp.pos64 = c->precision == TERSOFF_FP64 ? c->d_pos64 : nullptr;
+      bp.pos64 = c->d_pos64;
+      bp.fix64 = G.fix64;
+      bp.box = make_box64(G.L, G.fix64);
       bp.kmask = c->d_kmask;
-      TGB_CUDA(c, launch_pdl(k_bin_pack, nb, B, 0, s, n, x, g, bp, c->d_cell_of, c->d_cell_count,
-                             c->d_origin, c->d_qorg, c->d_flags));
+      TGB_CUDA(c, launch_pdl(c->precision == TERSOFF_FP64 ? k_bin_pack<true> : k_bin_pack<false>, nb, B, 0, s, n, x, g, bp, c->d_cell_of, c->d_cell_count,
+                             c->d_qorg, c->d_flags));
     }
   }
   const int m = (int)ncell + 1;

@@ -501,7 +501,7 @@ template <class T, int NS, bool BATCH>
 __global__ void __launch_bounds__(BwdBlock<T>::size) k_tersoff_bwd(const __grid_constant__ BwdArgs<T> a) {
   constexpr int SNS = NS > 0 ? NS : TERSOFF_MAX_SPECIES;
   __shared__ T sraw[SNS * SNS * SNS * NP];
-  __shared__ T sfilt[SNS * SNS];
+  __shared__ float sfilt[SNS * SNS];
   __shared__ double sgrad[SNS * SNS * SNS * NP];
   extern __shared__ __align__(16) unsigned char bwd_dyn[];
   T* slots = reinterpret_cast<T*>(bwd_dyn);
@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(BS) k_tersoff_hvp(const __grid_constant__ BwdA
                                                     double* __restrict__ gx, int b0, int b1) {
   constexpr int SNS = TERSOFF_MAX_SPECIES;
   __shared__ T sraw[SNS * SNS * SNS * NP];
-  __shared__ T sfilt[SNS * SNS];
+  __shared__ float sfilt[SNS * SNS];
   __shared__ int nb[3];
   extern __shared__ __align__(16) unsigned char hvp_dyn[];
   T* geo = reinterpret_cast<T*>(hvp_dyn);
@@ -1019,10 +1019,6 @@ __global__ void k_scale_forces(double* __restrict__ f, const double* __restrict_
   if (t < n3) f[t] = -gE[atom_sys ? atom_sys[t / 3] : 0] * f[t];
 }
 
-template <class T> const T* filt_ptr(Ctx* c);
-template <> inline const float* filt_ptr<float>(Ctx* c) { return c->d_filt32; }
-template <> inline const double* filt_ptr<double>(Ctx* c) { return c->d_filt64; }
-
 // force weights in T: the caller's doubles, or a float copy (mixed path)
 inline const double* weights_t(Ctx*, const double* gF, cudaStream_t, double*) { return gF; }
 inline const float* weights_t(Ctx* c, const double* gF, cudaStream_t s, float*) {
@@ -1049,11 +1045,11 @@ BwdArgs<T> make_args(Ctx* c, const T* raw, const double* gE, const double* gF, d
   g.types = c->d_types;
   g.pos32 = c->d_pos32;
   g.posq = c->d_posq;
-  g.pos64 = c->d_pos64;
-  g.filt2 = filt_ptr<T>(c);
+  g.filt2 = c->d_filt32;
+  fwd::set_pos64(c, g);
   const double scale = ldexp(1.0, c->grid.fix_shift);
   for (int q = 0; q < 3; ++q) {
-    g.h[q] = (T)c->grid.h[q];
+    g.h[q] = (float)c->grid.h[q];
     g.hq[q] = (int)llrint(c->grid.h[q] * scale);
   }
   g.qinv = ldexpf(1.0f, -c->grid.fix_shift);

@@ -29,6 +29,8 @@
 
 #include "fxmath.cuh"
 #include "internal.cuh"
+#include "pos64.cuh"
+#include "tersoff_fx.cuh"
 
 namespace tgb {
 namespace fwd {
@@ -163,7 +165,16 @@ __device__ __forceinline__ void small_real(int m, double& w) {
 }
 
 // ---------------------------------------------------------------- arguments
-template <class T> struct FwdArgs {
+// integer records of the FP64 path (tersoff_lanes64.cuh)
+template <class T> struct FxArgs {};
+template <> struct FxArgs<double> {
+  FxRec fx1;         // the record of a one-species table
+  const FxRec* fx;   // ns^3 records
+  int qd;            // fraction bits of the bond vectors
+  int cut_j;         // f_C(r_ik) does not depend on j
+};
+
+template <class T> struct FwdArgs : FxArgs<T> {
   int n, cap;
   int ns;                // species count (used when the kernel's NS is 0)
   const uint32_t* nbr;   // slot-major skin list
@@ -171,14 +182,18 @@ template <class T> struct FwdArgs {
   const int* types;
   const float4* pos32;   // mixed: (u, type bits)
   const int4* posq;      // mixed: fixed-point u, type
-  const dpos4* pos64;  // fp64: (u, type)
+  const ipos4* pos64;    // fp64: fixed-point position, type
+  int fix64;             // its scale 2^fix64
+  int coarse64;          // bits dropped for the float filter of its differences
+  float coarse_inv;      // ... and what one of the others is, in A
+  Box64 box;             // (single systems)
   const T* rec;          // ns^3 derived records
   T prm1[RSTRIDE];       // the record of a one-species table (read from the
                          // kernel-parameter constant bank)
-  const T* filt2;        // ns x ns squared filter radii
+  const float* filt2;    // ns x ns squared filter radii
   const float* near2;    // ns x ns: squared radii beyond which a bond gets its exact length
                          // residual (float path; unused by the double path)
-  T h[3];                // cell edges
+  float h[3];            // cell edges
   int hq[3];             // cell edges in fixed point
   float qinv;            // 2^-fix_shift
   const uint32_t* shortl;  // slot-major short list (filter radius + margin)
@@ -213,10 +228,22 @@ template <class T> struct FwdArgs {
                          // list's count (FLAG_LEFT) and its own ticket
 };
 
-// position of atom j relative to its origin, in T, and its species
+// The FP64 path's position format (host).
+template <class T> void set_pos64(const Ctx* c, FwdArgs<T>& a) {
+  a.pos64 = c->d_pos64;
+  a.fix64 = c->grid.fix64;
+  a.box = make_box64(c->grid.L, c->grid.fix64);
+  // differences of up to four list radii fit the filter's 32 bits
+  int keep = 30 - (int)ceil(log2(4.0 * c->r_list));
+  if (keep > c->grid.fix64) keep = c->grid.fix64;
+  a.coarse64 = c->grid.fix64 - keep;
+  a.coarse_inv = ldexpf(1.0f, -keep);
+}
+
+// position of atom j relative to its cell's origin in float (filter precision,
+// cheap), and its species
 template <class T> struct Pos;
 template <> struct Pos<float> {
-  // filter precision (cheap): float offsets
   static __device__ __forceinline__ void coarse(const FwdArgs<float>& a, int j, float& x,
                                                 float& y, float& z, int& t) {
     int4 p = __ldg(&a.posq[j]);
@@ -224,16 +251,6 @@ template <> struct Pos<float> {
     y = (float)p.y * a.qinv;
     z = (float)p.z * a.qinv;
     t = p.w;
-  }
-};
-template <> struct Pos<double> {
-  static __device__ __forceinline__ void coarse(const FwdArgs<double>& a, int j, double& x,
-                                                double& y, double& z, int& t) {
-    dpos4 p = a.pos64[j];
-    x = p.x;
-    y = p.y;
-    z = p.z;
-    t = get_int(p.w);
   }
 };
 
@@ -244,33 +261,37 @@ __device__ __forceinline__ void decode(uint32_t e, int& j, int& ox, int& oy, int
   oz = (int)(e >> 30) - 1;
 }
 
-// o h for o in {-1, 0, 1}, by the bits of h
-__device__ __forceinline__ double times_unit(int o, double h) {
-  const long long b = __double_as_longlong(h) ^ ((long long)(o & 2) << 62);
-  return o == 0 ? 0.0 : __longlong_as_double(b);
-}
-__device__ __forceinline__ float times_unit(int o, float h) { return (float)o * h; }
-
-// Periodic shift units of atom i: the launch-wide cell edges, or (batches of
-// systems) those of atom i's system, loaded once per atom.
+// Periodic shift units of atom i: the launch-wide ones, or (batches of
+// systems) those of atom i's system, loaded once per atom. Mixed path: the
+// list cells' edges; FP64 path: the box.
 template <class T, bool BATCH> struct Shift {
   __device__ __forceinline__ void load(const FwdArgs<T>&, int) {}
   __device__ __forceinline__ int hq(const FwdArgs<T>& a, int q) const { return a.hq[q]; }
-  __device__ __forceinline__ T h(const FwdArgs<T>& a, int q) const { return a.h[q]; }
+  __device__ __forceinline__ float h(const FwdArgs<T>& a, int q) const { return a.h[q]; }
+  __device__ __forceinline__ long long L(const FwdArgs<T>& a, int q) const { return a.box.L[q]; }
 };
-template <class T> struct Shift<T, true> {
+template <> struct Shift<float, true> {
   int hq_[3];
-  T h_[3];
-  __device__ __forceinline__ void load(const FwdArgs<T>& a, int i) {
+  float h_[3];
+  __device__ __forceinline__ void load(const FwdArgs<float>& a, int i) {
     const SysShift& s = a.sys[a.atom_sys[i]];
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
       hq_[q] = s.hq[q];
-      h_[q] = (T)s.h[q];
+      h_[q] = s.hf[q];
     }
   }
-  __device__ __forceinline__ int hq(const FwdArgs<T>&, int q) const { return hq_[q]; }
-  __device__ __forceinline__ T h(const FwdArgs<T>&, int q) const { return h_[q]; }
+  __device__ __forceinline__ int hq(const FwdArgs<float>&, int q) const { return hq_[q]; }
+  __device__ __forceinline__ float h(const FwdArgs<float>&, int q) const { return h_[q]; }
+};
+template <> struct Shift<double, true> {
+  long long L_[3];
+  __device__ __forceinline__ void load(const FwdArgs<double>& a, int i) {
+    const SysShift& s = a.sys[a.atom_sys[i]];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) L_[q] = s.box.L[q];
+  }
+  __device__ __forceinline__ long long L(const FwdArgs<double>&, int q) const { return L_[q]; }
 };
 
 // Accurate bond vector from i to entry e's image of j.
@@ -293,17 +314,70 @@ template <> struct Bond<float> {
   }
 };
 template <> struct Bond<double> {
+  // the bond vector as exact integers (scale 2^fix64)
+  template <bool B>
+  static __device__ __forceinline__ void fixed(const FwdArgs<double>& a, const Shift<double, B>& sh,
+                                               const ipos4& pi, uint32_t e, long long& dx,
+                                               long long& dy, long long& dz, int& j, int& tj) {
+    j = (int)(e & ENTRY_JMASK);
+    const ipos4 pj = a.pos64[j];
+    dx = nearest(pj.x - pi.x, sh.L(a, 0));
+    dy = nearest(pj.y - pi.y, sh.L(a, 1));
+    dz = nearest(pj.z - pi.z, sh.L(a, 2));
+    tj = (int)pj.w;
+  }
   template <bool B>
   static __device__ __forceinline__ void vec(const FwdArgs<double>& a, const Shift<double, B>& sh,
-                                             dpos4 pi, uint32_t e, double& dx, double& dy,
+                                             const ipos4& pi, uint32_t e, double& dx, double& dy,
                                              double& dz, int& j, int& tj) {
-    int ox, oy, oz;
+    long long ix, iy, iz;
+    fixed(a, sh, pi, e, ix, iy, iz, j, tj);
+    dx = fx::from_fixed(ix, a.fix64);
+    dy = fx::from_fixed(iy, a.fix64);
+    dz = fx::from_fixed(iz, a.fix64);
+  }
+};
+
+// Squared length of a fixed-point bond vector in float (filter precision: the
+// filter radii have 2e-6 to spare); far components saturate.
+__device__ __forceinline__ float coarse2(const FwdArgs<double>& a, long long dx, long long dy, long long dz) {
+  auto f = [&](long long d) {
+    long long v = d >> a.coarse64;
+    v = v > 0x7fffff00ll ? 0x7fffff00ll : (v < -0x7fffff00ll ? -0x7fffff00ll : v);
+    return (float)(int)v * a.coarse_inv;
+  };
+  const float x = f(dx), y = f(dy), z = f(dz);
+  return x * x + y * y + z * z;
+}
+
+// The filter of the lists by the cutoffs: squared float distance of atom i to
+// the image of j in entry e, and j's species.
+template <class T, bool BATCH> struct Filter;
+template <bool BATCH> struct Filter<float, BATCH> {
+  float x, y, z;
+  __device__ __forceinline__ Filter(const FwdArgs<float>& a, int i, int& ti) { Pos<float>::coarse(a, i, x, y, z, ti); }
+  __device__ __forceinline__ float r2(const FwdArgs<float>& a, const Shift<float, BATCH>& sh, uint32_t e, int& tj) const {
+    int j, ox, oy, oz;
     decode(e, j, ox, oy, oz);
-    dpos4 pj = a.pos64[j];
-    dx = (pj.x - pi.x) + times_unit(ox, sh.h(a, 0));
-    dy = (pj.y - pi.y) + times_unit(oy, sh.h(a, 1));
-    dz = (pj.z - pi.z) + times_unit(oz, sh.h(a, 2));
-    tj = get_int(pj.w);
+    float xj, yj, zj;
+    Pos<float>::coarse(a, j, xj, yj, zj, tj);
+    const float dx = (xj - x) + ox * sh.h(a, 0);
+    const float dy = (yj - y) + oy * sh.h(a, 1);
+    const float dz = (zj - z) + oz * sh.h(a, 2);
+    return dx * dx + dy * dy + dz * dz;
+  }
+};
+template <bool BATCH> struct Filter<double, BATCH> {
+  ipos4 p;
+  __device__ __forceinline__ Filter(const FwdArgs<double>& a, int i, int& ti) {
+    p = a.pos64[i];
+    ti = (int)p.w;
+  }
+  __device__ __forceinline__ float r2(const FwdArgs<double>& a, const Shift<double, BATCH>& sh, uint32_t e, int& tj) const {
+    long long dx, dy, dz;
+    int j;
+    Bond<double>::fixed(a, sh, p, e, dx, dy, dz, j, tj);
+    return coarse2(a, dx, dy, dz);
   }
 };
 
@@ -329,7 +403,7 @@ template <> struct Exact<float> {
 };
 template <> struct Exact<double> {
   template <bool B>
-  static __device__ double residual(const FwdArgs<double>&, const Shift<double, B>&, dpos4,
+  static __device__ double residual(const FwdArgs<double>&, const Shift<double, B>&, const ipos4&,
                                     uint32_t, double) {
     return 0.0;
   }
@@ -339,7 +413,7 @@ constexpr float NEAR_CUT = 2e-3f;
 
 template <class T> struct SelfPos;
 template <> struct SelfPos<float> { using type = int4; };
-template <> struct SelfPos<double> { using type = dpos4; };
+template <> struct SelfPos<double> { using type = ipos4; };
 
 template <class T>
 __device__ __forceinline__ typename SelfPos<T>::type self_pos(const FwdArgs<T>& a, int i);
@@ -348,7 +422,7 @@ __device__ __forceinline__ int4 self_pos<float>(const FwdArgs<float>& a, int i) 
   return __ldg(&a.posq[i]);
 }
 template <>
-__device__ __forceinline__ dpos4 self_pos<double>(const FwdArgs<double>& a, int i) {
+__device__ __forceinline__ ipos4 self_pos<double>(const FwdArgs<double>& a, int i) {
   return a.pos64[i];
 }
 
@@ -794,7 +868,7 @@ template <class T> struct Acc<T, true> {
 // scattered with FP64 atomics (the TERSOFF_ABLATE_COMP_ATOM_SUMS variant).
 // Resident blocks per SM that the force kernel's launch bound asks for: the
 // register budget, and the grid of the "waves" launch option.
-// The FP64 instances run on the FP64 pipe (about 87% busy on the benchmark):
+// The FP64 instances (tables outside the integer formats) run on the FP64 pipe:
 // four blocks per SM give them 128 registers and no spills.
 __host__ __device__ constexpr int fwd_min_blocks(int zc, int ev, bool dbl = false) {
   return zc <= 4 ? (dbl ? 4 : (ev == 2 ? 7 : 8)) : 4;
@@ -813,7 +887,7 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
   constexpr int SNS = NS > 1 ? NS : (NS == 1 ? 1 : TERSOFF_MAX_SPECIES);
   constexpr int SREC = NS == 1 ? 1 : SNS * SNS * SNS * RSTRIDE;
   __shared__ T srec_s[SREC];
-  __shared__ T sfilt[SNS * SNS];
+  __shared__ float sfilt[SNS * SNS];
   const int ns = NS > 0 ? NS : a.ns;
   // launch-uniform words, read once per block (one load per lane, together)
   __shared__ int uni[5];
@@ -903,22 +977,13 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
       } else if (z_list > ZC) {
         // more stored entries than registers: keep those inside the cutoffs now
         filtered = true;
-        T xi, yi, zi;
         int tii;
-        Pos<T>::coarse(a, i, xi, yi, zi, tii);
+        const Filter<T, BATCH> flt(a, i, tii);
         const bool fits = z_list <= 64;
         if (fits)
           for (int s = 0; s < z_list; ++s) {
-            const uint32_t e = a.shortl[(size_t)s * a.n + i];
-            int j, ox, oy, oz;
-            decode(e, j, ox, oy, oz);
-            T xj, yj, zj;
             int tj;
-            Pos<T>::coarse(a, j, xj, yj, zj, tj);
-            const T dx = (xj - xi) + times_unit(ox, sh.h(a, 0));
-            const T dy = (yj - yi) + times_unit(oy, sh.h(a, 1));
-            const T dz = (zj - zi) + times_unit(oz, sh.h(a, 2));
-            const T r2 = dx * dx + dy * dy + dz * dz;
+            const float r2 = flt.r2(a, sh, a.shortl[(size_t)s * a.n + i], tj);
             if (r2 <= sfilt[ti * ns + tj]) mask |= 1ull << s;
           }
         z = __popcll(mask);
@@ -928,26 +993,16 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
     } else {
       // filter the skin list into a bit mask (Sec. IV-D)
       filtered = true;
-      T xi, yi, zi;
-      Pos<T>::coarse(a, i, xi, yi, zi, ti);
+      const Filter<T, BATCH> flt(a, i, ti);
       c = min(a.cnt[i], a.cap);
       list = a.nbr;
       const bool fits = c <= 64;
-      if (fits) {
+      if (fits)
         for (int s = 0; s < c; ++s) {
-          const uint32_t e = a.nbr[(size_t)s * a.n + i];
-          int j, ox, oy, oz;
-          decode(e, j, ox, oy, oz);
-          T xj, yj, zj;
           int tj;
-          Pos<T>::coarse(a, j, xj, yj, zj, tj);
-          const T dx = (xj - xi) + times_unit(ox, sh.h(a, 0));
-          const T dy = (yj - yi) + times_unit(oy, sh.h(a, 1));
-          const T dz = (zj - zi) + times_unit(oz, sh.h(a, 2));
-          const T r2 = dx * dx + dy * dy + dz * dz;
+          const float r2 = flt.r2(a, sh, a.nbr[(size_t)s * a.n + i], tj);
           if (r2 <= sfilt[ti * ns + tj]) mask |= 1ull << s;
         }
-      }
       z = __popcll(mask);
       general = !fits || z > ZC || a.all_general;
       have_mask = fits;
@@ -1243,7 +1298,7 @@ __global__ void __launch_bounds__(WIDE_BLOCK) k_tersoff_wide(const __grid_consta
   constexpr int SNS = NS > 1 ? NS : (NS == 1 ? 1 : TERSOFF_MAX_SPECIES);
   constexpr int SREC = NS == 1 ? 1 : SNS * SNS * SNS * RSTRIDE;
   __shared__ T srec_s[SREC];
-  __shared__ T sfilt[SNS * SNS];
+  __shared__ float sfilt[SNS * SNS];
   __shared__ int uni[3];
   extern __shared__ __align__(16) unsigned char wide_dyn[];
   T* sl = reinterpret_cast<T*>(wide_dyn);
