@@ -904,6 +904,102 @@ static int enqueue_md(Ctx* c, double* x, double* v, double* f, double dt,
   return TERSOFF_OK;
 }
 
+// After a build inside a call's sequence overflowed (or met non-finite
+// positions): restores the call's start state from the snapshot, rebuilds with
+// a host check and runs the steps eagerly.
+static int md_rerun(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
+                    double* rows, double* thermo, int ssb0, cudaStream_t s) {
+  const size_t m = 3 * (size_t)c->n;
+  const bool on_skin = rebuild_every == TERSOFF_REBUILD_ON_SKIN;
+  int st;
+  TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+  TGB_CUDA(c, cudaMemcpyAsync(v, c->d_snap + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+  TGB_CUDA(c, cudaMemcpyAsync(f, c->d_snap + 2 * m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+  if (c->h_flags[tgb::FLAG_NONFINITE]) {
+    if (!on_skin) c->steps_since_build = ssb0;
+    TGB_CUDA(c, cudaStreamSynchronize(s));
+    return tgb::fail(c, TERSOFF_E_NONFINITE, "non-finite position during MD (state restored)");
+  }
+  c->cap = c->cap + c->cap / 2 + 4;
+  c->gen++;
+  if ((st = tgb::build_list(c, x, s))) return st;
+  c->last_rebuilds = 0;
+  st = enqueue_md(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, true, s);
+  if (st) return st;
+  TGB_CUDA(c, cudaStreamSynchronize(s));
+  return TERSOFF_OK;
+}
+
+// The steps of a small system by the resident kernel (md_resident.cu): one
+// launch per stretch between rebuilds. With displacement-triggered rebuilds
+// the host reads where a launch ended; a fixed period needs no reading.
+constexpr int RESIDENT_STEPS = 4096;
+static int md_resident(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
+                       double* rows, double* thermo, cudaStream_t s) {
+  int st;
+  const bool on_skin = rebuild_every == TERSOFF_REBUILD_ON_SKIN;
+  const int ssb0 = c->steps_since_build;
+  if (rows) TGB_CUDA(c, cudaMemsetAsync(rows, 0, sizeof(double) * tgb::ACC_LEN * (size_t)nsteps, s));
+  int done = 0;         // the next launch's first step
+  bool resume = false;  // ... has been drifted
+  for (;;) {
+    int s1 = nsteps;
+    bool tail = false;
+    if (rebuild_every > 0) {
+      const int left = rebuild_every - c->steps_since_build;
+      const long long at = (long long)done + (resume ? 1 : 0) + (left > 1 ? left : 1) - 1;
+      if (at < nsteps) {
+        s1 = (int)at;
+        tail = true;
+      }
+    }
+    // (a bound on the time one launch takes)
+    const bool more = s1 - done > RESIDENT_STEPS;
+    if (more) {
+      s1 = done + RESIDENT_STEPS;
+      tail = false;
+    }
+    if ((st = tgb::launch_resident(c, x, v, f, dt, done, s1, resume, tail, on_skin, skin_lim2(c), rows, c->d_snap, s)))
+      return st;
+    if (!on_skin && (more || !tail)) c->steps_since_build += s1 - done - (resume ? 1 : 0);
+    bool halted = false;
+    if (on_skin) {
+      if ((st = tgb::read_flags(c, s))) return st;
+      if (c->h_flags[tgb::FLAG_MD_TIMEOUT] || c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE]) break;
+      halted = c->h_flags[tgb::FLAG_MD_HALT] != 0;
+      if (halted) s1 = c->h_flags[tgb::FLAG_MD_STEP];
+    }
+    done = s1;
+    resume = halted || tail;
+    if (resume) {
+      if ((st = tgb::build_list_async(c, x, s))) return st;
+      if (!on_skin) c->steps_since_build = 0;
+      c->last_rebuilds++;
+    } else if (!more) {
+      break;
+    }
+  }
+  double* ke_row = rows ? rows + tgb::ACC_LEN * (size_t)(nsteps - 1) + 7 * tgb::ACC_STRIDE : nullptr;
+  if ((st = tgb::launch_final_kick(c, v, f, ke_row, s))) return st;
+  if (thermo && (st = tgb::launch_thermo_rows(c, rows, nsteps, tgb::MVV2E, thermo, s))) return st;
+  if ((st = tgb::read_flags(c, s))) return st;
+  if (c->h_flags[tgb::FLAG_MD_TIMEOUT]) {
+    const size_t m = 3 * (size_t)c->n;
+    TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    TGB_CUDA(c, cudaMemcpyAsync(v, c->d_snap + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    TGB_CUDA(c, cudaMemcpyAsync(f, c->d_snap + 2 * m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
+    TGB_CUDA(c, cudaStreamSynchronize(s));
+    c->have_list = false;
+    return tgb::fail(c, TERSOFF_E_TIMEOUT, "a wait between MD steps gave up (state restored; rebuild the list)");
+  }
+  if (c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE])
+    return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, on_skin ? c->steps_since_build : ssb0, s);
+  c->max_cnt = c->h_flags[tgb::FLAG_OVERFLOW];
+  c->max_short = c->h_flags[tgb::FLAG_SHORT_MAX];
+  for (int b = 0; b < 3; ++b) c->nbucket[b] = c->h_flags[tgb::flag_bucket(b)];
+  return TERSOFF_OK;
+}
+
 static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double* mass,
                    double dt, int nsteps, int rebuild_every, double* thermo, cudaStream_t s) {
   if (c) c->fine_valid = false;  // the steps may rebuild the lists on the device
@@ -961,6 +1057,8 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     if ((st = tgb::dev_alloc(c, &c->d_snap, 3 * m))) return st;
     c->snap_alloc = 3 * m;
   }
+  if (!c->timing && tgb::resident_fits(c, rows != nullptr))
+    return md_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, s);
   const int ssb0 = on_skin ? -1 : c->steps_since_build;
   auto& G = c->graph;
   const bool same = G.exec && G.gen == c->gen && G.x == x && G.v == v && G.f == f &&
@@ -1045,24 +1143,7 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     for (int b = 0; b < 3; ++b) c->nbucket[b] = c->h_flags[tgb::flag_bucket(b)];
     return TERSOFF_OK;
   }
-  // a build inside the sequence overflowed (or met non-finite positions):
-  // restore the state, rebuild with a host check, run the steps eagerly
-  TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-  TGB_CUDA(c, cudaMemcpyAsync(v, c->d_snap + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-  TGB_CUDA(c, cudaMemcpyAsync(f, c->d_snap + 2 * m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-  if (c->h_flags[tgb::FLAG_NONFINITE]) {
-    if (!on_skin) c->steps_since_build = ssb0;
-    TGB_CUDA(c, cudaStreamSynchronize(s));
-    return tgb::fail(c, TERSOFF_E_NONFINITE, "non-finite position during MD (state restored)");
-  }
-  c->cap = c->cap + c->cap / 2 + 4;
-  c->gen++;
-  if ((st = tgb::build_list(c, x, s))) return st;
-  c->last_rebuilds = 0;
-  st = enqueue_md(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, true, s);
-  if (st) return st;
-  TGB_CUDA(c, cudaStreamSynchronize(s));
-  return TERSOFF_OK;
+  return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
 }
 
 int tersoff_md_step(tersoff_ctx* p, double* x, double* v, double* f, int n, const double* mass,

@@ -10,6 +10,8 @@ int launch_forward_f32(Ctx* c, double* f, double* acc, double* eatom, cudaStream
     default: return fwd::launch_species<float, 0>(c, f, acc, eatom, s, virial);
   }
 }
+fwd::FwdArgs<float> resident_args(Ctx* c) { return fwd::make_args<float>(c, c->d_extra, nullptr, nullptr, false); }
+
 int launch_forward_batch_f32(Ctx* c, double* f, cudaStream_t s) {
   return fwd::launch_batch<float>(c, f, s);
 }

@@ -353,7 +353,11 @@ enum : int {
   FLAG_LEFT = 14 * FLAG_STRIDE,         // atoms the four-lane force kernel left to the
                                         // per-thread kernel (0 between evaluations)
   FLAG_LEFT_TICKET = 15 * FLAG_STRIDE,  // blocks of that per-thread launch done (0 between)
-  FLAG_COUNT = 16 * FLAG_STRIDE
+  FLAG_MD_STEP = 16 * FLAG_STRIDE,      // resident MD kernel: the step it ended at,
+  FLAG_MD_HALT = 17 * FLAG_STRIDE,      // ... 1: for a displacement-triggered rebuild,
+  FLAG_MD_BAR = 18 * FLAG_STRIDE,       // ... its barrier's arrivals (after the halt word),
+  FLAG_MD_TIMEOUT = 19 * FLAG_STRIDE,   // ... 1: a bounded wait gave up
+  FLAG_COUNT = 20 * FLAG_STRIDE
 };
 __host__ __device__ constexpr int flag_bucket(int b) { return FLAG_BUCKET + b * FLAG_STRIDE; }
 
@@ -475,6 +479,20 @@ int launch_decide_rebuild(Ctx* c, float lim2, cudaGraphConditionalHandle h, cuda
 int launch_halo_pack(Ctx* c, const double* x, const int* types, const long long* ids, int n,
                      int axis, const double* geo, int cap, double* x_local, double* send_x,
                      int* send_t, long long* send_id, int* counts, cudaStream_t s);
+
+// Resident MD kernel of small systems (md_resident.cu). resident_fits: whether
+// the context's steps run in it (rows: with thermo accumulation).
+// launch_resident: steps s0 .. s1 - 1 (resume: from the forces of s0, whose
+// drift ran before a rebuild; tail: then the drift of s1 before a rebuild);
+// with on_skin the kernel ends at the first step whose displacement asks for a
+// rebuild. Its end is in the FLAG_MD_* words.
+// The size limit: 512 blocks of 128 fit the chip at once, and the launches'
+// share of a step has shrunk (on-skin steps at 64,000 atoms 23.1 us resident,
+// 33.1 at 110,592 as graph nodes).
+constexpr int RESIDENT_MAX_ATOMS = 65536;
+bool resident_fits(Ctx* c, bool rows);
+int launch_resident(Ctx* c, double* x, double* v, const double* f, double dt, int s0, int s1, bool resume, bool tail,
+                    bool on_skin, float lim2, double* rows, double* snap, cudaStream_t s);
 
 int launch_thermo_rows(Ctx* c, const double* rows, int nsteps, double mvv2e, double* thermo,
                        cudaStream_t s);

@@ -246,7 +246,9 @@ template <class T> struct Pos;
 template <> struct Pos<float> {
   static __device__ __forceinline__ void coarse(const FwdArgs<float>& a, int j, float& x,
                                                 float& y, float& z, int& t) {
-    int4 p = __ldg(&a.posq[j]);
+    offsets(a, __ldg(&a.posq[j]), x, y, z, t);
+  }
+  static __device__ __forceinline__ void offsets(const FwdArgs<float>& a, int4 p, float& x, float& y, float& z, int& t) {
     x = (float)p.x * a.qinv;
     y = (float)p.y * a.qinv;
     z = (float)p.z * a.qinv;
@@ -263,14 +265,19 @@ __device__ __forceinline__ void decode(uint32_t e, int& j, int& ox, int& oy, int
 
 // Periodic shift units of atom i: the launch-wide ones, or (batches of
 // systems) those of atom i's system, loaded once per atom. Mixed path: the
-// list cells' edges; FP64 path: the box.
-template <class T, bool BATCH> struct Shift {
+// list cells' edges; FP64 path: the box. KIND: 0 one system, 1 a batch, 2 one
+// system whose positions change while the kernel runs (the resident MD loop):
+// their loads must not go through the read-only path.
+template <class T, int KIND> struct Shift {
   __device__ __forceinline__ void load(const FwdArgs<T>&, int) {}
   __device__ __forceinline__ int hq(const FwdArgs<T>& a, int q) const { return a.hq[q]; }
   __device__ __forceinline__ float h(const FwdArgs<T>& a, int q) const { return a.h[q]; }
   __device__ __forceinline__ long long L(const FwdArgs<T>& a, int q) const { return a.box.L[q]; }
+  __device__ __forceinline__ int4 posq(const FwdArgs<T>& a, int j) const {
+    return KIND == 2 ? a.posq[j] : __ldg(&a.posq[j]);
+  }
 };
-template <> struct Shift<float, true> {
+template <> struct Shift<float, 1> {
   int hq_[3];
   float h_[3];
   __device__ __forceinline__ void load(const FwdArgs<float>& a, int i) {
@@ -283,8 +290,9 @@ template <> struct Shift<float, true> {
   }
   __device__ __forceinline__ int hq(const FwdArgs<float>&, int q) const { return hq_[q]; }
   __device__ __forceinline__ float h(const FwdArgs<float>&, int q) const { return h_[q]; }
+  __device__ __forceinline__ int4 posq(const FwdArgs<float>& a, int j) const { return __ldg(&a.posq[j]); }
 };
-template <> struct Shift<double, true> {
+template <> struct Shift<double, 1> {
   long long L_[3];
   __device__ __forceinline__ void load(const FwdArgs<double>& a, int i) {
     const SysShift& s = a.sys[a.atom_sys[i]];
@@ -297,13 +305,13 @@ template <> struct Shift<double, true> {
 // Accurate bond vector from i to entry e's image of j.
 template <class T> struct Bond;
 template <> struct Bond<float> {
-  template <bool B>
+  template <int B>
   static __device__ __forceinline__ void vec(const FwdArgs<float>& a, const Shift<float, B>& sh,
                                              int4 qi, uint32_t e, float& dx, float& dy,
                                              float& dz, int& j, int& tj) {
     int ox, oy, oz;
     decode(e, j, ox, oy, oz);
-    int4 qj = __ldg(&a.posq[j]);
+    int4 qj = sh.posq(a, j);
     int ix = qj.x - qi.x + ox * sh.hq(a, 0);
     int iy = qj.y - qi.y + oy * sh.hq(a, 1);
     int iz = qj.z - qi.z + oz * sh.hq(a, 2);
@@ -315,7 +323,7 @@ template <> struct Bond<float> {
 };
 template <> struct Bond<double> {
   // the bond vector as exact integers (scale 2^fix64)
-  template <bool B>
+  template <int B>
   static __device__ __forceinline__ void fixed(const FwdArgs<double>& a, const Shift<double, B>& sh,
                                                const ipos4& pi, uint32_t e, long long& dx,
                                                long long& dy, long long& dz, int& j, int& tj) {
@@ -326,7 +334,7 @@ template <> struct Bond<double> {
     dz = nearest(pj.z - pi.z, sh.L(a, 2));
     tj = (int)pj.w;
   }
-  template <bool B>
+  template <int B>
   static __device__ __forceinline__ void vec(const FwdArgs<double>& a, const Shift<double, B>& sh,
                                              const ipos4& pi, uint32_t e, double& dx, double& dy,
                                              double& dz, int& j, int& tj) {
@@ -352,24 +360,26 @@ __device__ __forceinline__ float coarse2(const FwdArgs<double>& a, long long dx,
 
 // The filter of the lists by the cutoffs: squared float distance of atom i to
 // the image of j in entry e, and j's species.
-template <class T, bool BATCH> struct Filter;
-template <bool BATCH> struct Filter<float, BATCH> {
+template <class T, int BATCH> struct Filter;
+template <int BATCH> struct Filter<float, BATCH> {
   float x, y, z;
-  __device__ __forceinline__ Filter(const FwdArgs<float>& a, int i, int& ti) { Pos<float>::coarse(a, i, x, y, z, ti); }
+  __device__ __forceinline__ Filter(const FwdArgs<float>& a, const Shift<float, BATCH>& sh, int i, int& ti) {
+    Pos<float>::offsets(a, sh.posq(a, i), x, y, z, ti);
+  }
   __device__ __forceinline__ float r2(const FwdArgs<float>& a, const Shift<float, BATCH>& sh, uint32_t e, int& tj) const {
     int j, ox, oy, oz;
     decode(e, j, ox, oy, oz);
     float xj, yj, zj;
-    Pos<float>::coarse(a, j, xj, yj, zj, tj);
+    Pos<float>::offsets(a, sh.posq(a, j), xj, yj, zj, tj);
     const float dx = (xj - x) + ox * sh.h(a, 0);
     const float dy = (yj - y) + oy * sh.h(a, 1);
     const float dz = (zj - z) + oz * sh.h(a, 2);
     return dx * dx + dy * dy + dz * dz;
   }
 };
-template <bool BATCH> struct Filter<double, BATCH> {
+template <int BATCH> struct Filter<double, BATCH> {
   ipos4 p;
-  __device__ __forceinline__ Filter(const FwdArgs<double>& a, int i, int& ti) {
+  __device__ __forceinline__ Filter(const FwdArgs<double>& a, const Shift<double, BATCH>&, int i, int& ti) {
     p = a.pos64[i];
     ti = (int)p.w;
   }
@@ -386,12 +396,12 @@ template <bool BATCH> struct Filter<double, BATCH> {
 // double path's r is already accurate to rounding: 0).
 template <class T> struct Exact;
 template <> struct Exact<float> {
-  template <bool B>
+  template <int B>
   static __device__ float residual(const FwdArgs<float>& a, const Shift<float, B>& sh, int4 qi,
                                    uint32_t e, float r) {
     int j, ox, oy, oz;
     decode(e, j, ox, oy, oz);
-    const int4 qj = __ldg(&a.posq[j]);
+    const int4 qj = sh.posq(a, j);
     const long long ix = qj.x - qi.x + ox * sh.hq(a, 0);
     const long long iy = qj.y - qi.y + oy * sh.hq(a, 1);
     const long long iz = qj.z - qi.z + oz * sh.hq(a, 2);
@@ -402,7 +412,7 @@ template <> struct Exact<float> {
   }
 };
 template <> struct Exact<double> {
-  template <bool B>
+  template <int B>
   static __device__ double residual(const FwdArgs<double>&, const Shift<double, B>&, const ipos4&,
                                     uint32_t, double) {
     return 0.0;
@@ -417,6 +427,14 @@ template <> struct SelfPos<double> { using type = ipos4; };
 
 template <class T>
 __device__ __forceinline__ typename SelfPos<T>::type self_pos(const FwdArgs<T>& a, int i);
+template <int B>
+__device__ __forceinline__ int4 self_pos(const FwdArgs<float>& a, const Shift<float, B>& sh, int i) {
+  return sh.posq(a, i);
+}
+template <int B>
+__device__ __forceinline__ ipos4 self_pos(const FwdArgs<double>& a, const Shift<double, B>&, int i) {
+  return a.pos64[i];
+}
 template <>
 __device__ __forceinline__ int4 self_pos<float>(const FwdArgs<float>& a, int i) {
   return __ldg(&a.posq[i]);
@@ -585,7 +603,7 @@ __device__ __forceinline__ int rec_off(int ns, int ti, int tj, int tk) {
 // use_mask: bit s of mask marks the entries s < 64 inside the filter radius
 // (the others cannot be in any term and are skipped before their bond vector
 // is formed).
-template <class T, int NS, bool LAM3, bool BATCH>
+template <class T, int NS, bool LAM3, int BATCH>
 __device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T, BATCH>& sh,
                                           const T* srec, int i, int ti,
                                           const uint32_t* list, int c, bool slots,
@@ -593,7 +611,7 @@ __device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T,
                                           T* w) {
   using P = typename SelfPos<T>::type;
   const int ns = NS > 0 ? NS : a.ns;
-  const P pi = self_pos<T>(a, i);
+  const P pi = self_pos(a, sh, i);
   T fix = 0, fiy = 0, fiz = 0;
   // exact length residual of a bond near a cutoff (float path)
   auto near_res = [&](uint32_t e, T r2, T r, int tx) -> T {
@@ -874,69 +892,40 @@ __host__ __device__ constexpr int fwd_min_blocks(int zc, int ev, bool dbl = fals
   return zc <= 4 ? (dbl ? 4 : (ev == 2 ? 7 : 8)) : 4;
 }
 
+// What every atom of a launch shares.
+template <class T> struct ItemEnv {
+  const T* srec;        // derived records
+  const float* sfilt;   // squared filter radii
+  const float* snear;
+  int ns;
+  int n_first, n_second, n_items;  // items of the launch's up to three orders
+  bool slots, use_short, want_acc;
+  typename SumT<T>::type* tsum;    // this thread's energy and virial sums (stride BLOCK)
+};
+
 // EV: 2 energy and virial (and per-atom energy) as requested; 1 energy and
 // per-atom energy only (the MD steps' thermo); 0 forces only (the MD steps
 // without thermo). Instances 0 and 1 carry less bookkeeping and fit one more
 // block per SM.
-template <class T, int NS, int ZC, int MODE, bool BATCH = false, bool CS = false, int EV = 2>
-__global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
-    k_tersoff(const __grid_constant__ FwdArgs<T> a) {
-  static_assert(!(CS && BATCH), "compensated per-atom sums: single systems only");
-  static_assert(EV == 2 || !BATCH, "batches need the per-atom energy and virial");
-  pdl_wait();  // the previous kernel's writes (a launch with launch_pdl)
-  constexpr int SNS = NS > 1 ? NS : (NS == 1 ? 1 : TERSOFF_MAX_SPECIES);
-  constexpr int SREC = NS == 1 ? 1 : SNS * SNS * SNS * RSTRIDE;
-  __shared__ T srec_s[SREC];
-  __shared__ float sfilt[SNS * SNS];
-  const int ns = NS > 0 ? NS : a.ns;
-  // launch-uniform words, read once per block (one load per lane, together)
-  __shared__ int uni[5];
-  __shared__ float snear[SNS * SNS];
-  if (NS != 1)
-    for (int q = threadIdx.x; q < ns * ns * ns * RSTRIDE; q += BLOCK) srec_s[q] = a.rec[q];
-  if (threadIdx.x < ns * ns) {
-    sfilt[threadIdx.x] = a.filt2[threadIdx.x];
-    snear[threadIdx.x] = sizeof(T) == 4 ? a.near2[threadIdx.x] : 0.0f;
-  }
-  if (threadIdx.x < 5) {
-    const int* src = threadIdx.x == 0   ? a.n_items
-                     : threadIdx.x == 1 ? a.flags + FLAG_REV_MISS
-                     : threadIdx.x == 2 ? a.flags + FLAG_DMAX
-                     : threadIdx.x == 3 ? a.n_items2
-                                        : a.n_items3;
-    uni[threadIdx.x] = src ? *src : 0;
-  }
-  __syncthreads();
-  // parameters: shared memory for several species (type-dependent records),
-  // the constant bank for one species (uniform, operands of the FP instructions)
-  const T* srec = NS == 1 ? a.prm1 : srec_s;
+// The items item, item + stride, ... of one thread; returns whether it had any.
+template <class T, int NS, int ZC, int MODE, int BATCH, bool CS, int EV>
+__device__ __forceinline__ bool force_items(const FwdArgs<T>& a, const ItemEnv<T>& v, int item, int stride) {
   constexpr bool LAM3 = MODE == 1;
-  const int n_first = uni[0];
-  const int n_second = uni[0] + uni[3];
-  const int n_items = a.identity ? a.n : min(n_second + uni[4], a.n);
-  // slots: contributions go to per-slot stores (needs the stored short list and
-  // its reverse map); otherwise FP64 atomics into the fallback buffer
-  const bool slots_ok = uni[1] == 0;
-  // the stored short list holds every atom that can be inside a cutoff while no
-  // atom has moved more than half the list margin since the build (uniform)
-  const bool use_short = __int_as_float(uni[2]) <= a.dlim2;
-  const bool slots = !a.atomic_mode && use_short && slots_ok;
-  if (blockIdx.x == 0 && threadIdx.x == 0) a.flags[FLAG_EXTRA] = slots ? 0 : 1;
-  // the atom's own virial sums (float), and the thread's energy and virial
-  // over its atoms in double, kept in the thread's column of a shared-memory
-  // table (not in registers) and formed only when the reduction is wanted
+  const int ns = NS > 0 ? NS : v.ns;
+  const T* const srec = v.srec;
+  const float* const sfilt = v.sfilt;
+  const float* const snear = v.snear;
+  const bool slots = v.slots, use_short = v.use_short, want_acc = v.want_acc;
+  // the atom's own virial sums; those over the thread's atoms stay in its
+  // column of a shared-memory table (not in registers), formed only when the
+  // reduction is wanted
   T w[6];
-  __shared__ typename SumT<T>::type tsum[7][BLOCK];
-  const bool want_acc = a.acc != nullptr;
-  if (want_acc)
-    for (int q = 0; q < 7; ++q) sum_zero(tsum[q][threadIdx.x]);
   bool any = false;
-  for (int item = blockIdx.x * BLOCK + threadIdx.x; item < n_items;
-       item += gridDim.x * BLOCK) {
+  for (; item < v.n_items; item += stride) {
     any = true;
     const int i = a.identity ? item
-                  : (item < n_first ? a.order[item]
-                     : (item < n_second ? a.order2[item - n_first] : a.order3[item - n_second]));
+                  : (item < v.n_first ? a.order[item]
+                     : (item < v.n_second ? a.order2[item - v.n_first] : a.order3[item - v.n_second]));
     T eatom_i = T(0);
     Acc<T, CS> eatom_c;  // CS: the atom's energy (fast path)
     Acc<T, CS> wa[6];    // CS: the atom's virial (fast path)
@@ -953,7 +942,7 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
     bool have_mask = false; // mask covers every entry of list (at most 64)
     int z_list = 0;         // stored short-list length (slots mode bookkeeping)
     using P = typename SelfPos<T>::type;
-    const P pi = self_pos<T>(a, i);
+    const P pi = self_pos(a, sh, i);
     // the first ZC stored entries and their reverse slots (for the scatter),
     // loaded together with the count: every atom has at least 8 list slots, so
     // they are in bounds whatever the count
@@ -978,7 +967,7 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
         // more stored entries than registers: keep those inside the cutoffs now
         filtered = true;
         int tii;
-        const Filter<T, BATCH> flt(a, i, tii);
+        const Filter<T, BATCH> flt(a, sh, i, tii);
         const bool fits = z_list <= 64;
         if (fits)
           for (int s = 0; s < z_list; ++s) {
@@ -993,7 +982,7 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
     } else {
       // filter the skin list into a bit mask (Sec. IV-D)
       filtered = true;
-      const Filter<T, BATCH> flt(a, i, ti);
+      const Filter<T, BATCH> flt(a, sh, i, ti);
       c = min(a.cnt[i], a.cap);
       list = a.nbr;
       const bool fits = c <= 64;
@@ -1248,11 +1237,11 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
       // compensated ones (eatom_c, wa), into the thread's double sums
       if (a.eatom) a.eatom[i] = to_f64(eatom_i) + eatom_c.d();
       if (want_acc) {
-        sum_add(tsum[0][threadIdx.x], eatom_i);
-        sum_add2(tsum[0][threadIdx.x], eatom_c.s, eatom_c.lo());
+        sum_add(v.tsum[0], eatom_i);
+        sum_add2(v.tsum[0], eatom_c.s, eatom_c.lo());
         for (int q = 0; q < 6; ++q) {
-          sum_add(tsum[1 + q][threadIdx.x], w[q]);
-          sum_add2(tsum[1 + q][threadIdx.x], wa[q].s, wa[q].lo());
+          sum_add(v.tsum[(1 + q) * BLOCK], w[q]);
+          sum_add2(v.tsum[(1 + q) * BLOCK], wa[q].s, wa[q].lo());
         }
       }
       continue;
@@ -1261,13 +1250,67 @@ __global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
     eatom_i += eatom_c.s;
     if (a.eatom) a.eatom[i] = to_f64(eatom_i);
     if (want_acc) {
-      sum_add(tsum[0][threadIdx.x], eatom_i);
+      sum_add(v.tsum[0], eatom_i);
       if (EV == 2)
-        for (int q = 0; q < 6; ++q) sum_add(tsum[1 + q][threadIdx.x], w[q]);
+        for (int q = 0; q < 6; ++q) sum_add(v.tsum[(1 + q) * BLOCK], w[q]);
     }
-    if (BATCH)
+    if (BATCH == 1)
       for (int q = 0; q < 6; ++q) a.vatom[6 * (size_t)i + q] = to_f64(w[q]);
   }
+  return any;
+}
+
+template <class T, int NS, int ZC, int MODE, bool BATCH = false, bool CS = false, int EV = 2>
+__global__ void __launch_bounds__(BLOCK, fwd_min_blocks(ZC, EV, sizeof(T) == 8))
+    k_tersoff(const __grid_constant__ FwdArgs<T> a) {
+  static_assert(!(CS && BATCH), "compensated per-atom sums: single systems only");
+  static_assert(EV == 2 || !BATCH, "batches need the per-atom energy and virial");
+  pdl_wait();  // the previous kernel's writes (a launch with launch_pdl)
+  constexpr int SNS = NS > 1 ? NS : (NS == 1 ? 1 : TERSOFF_MAX_SPECIES);
+  constexpr int SREC = NS == 1 ? 1 : SNS * SNS * SNS * RSTRIDE;
+  __shared__ T srec_s[SREC];
+  __shared__ float sfilt[SNS * SNS];
+  const int ns = NS > 0 ? NS : a.ns;
+  // launch-uniform words, read once per block (one load per lane, together)
+  __shared__ int uni[5];
+  __shared__ float snear[SNS * SNS];
+  if (NS != 1)
+    for (int q = threadIdx.x; q < ns * ns * ns * RSTRIDE; q += BLOCK) srec_s[q] = a.rec[q];
+  if (threadIdx.x < ns * ns) {
+    sfilt[threadIdx.x] = a.filt2[threadIdx.x];
+    snear[threadIdx.x] = sizeof(T) == 4 ? a.near2[threadIdx.x] : 0.0f;
+  }
+  if (threadIdx.x < 5) {
+    const int* src = threadIdx.x == 0   ? a.n_items
+                     : threadIdx.x == 1 ? a.flags + FLAG_REV_MISS
+                     : threadIdx.x == 2 ? a.flags + FLAG_DMAX
+                     : threadIdx.x == 3 ? a.n_items2
+                                        : a.n_items3;
+    uni[threadIdx.x] = src ? *src : 0;
+  }
+  __syncthreads();
+  // parameters: shared memory for several species (type-dependent records),
+  // the constant bank for one species (uniform, operands of the FP instructions)
+  const T* srec = NS == 1 ? a.prm1 : srec_s;
+  const int n_first = uni[0];
+  const int n_second = uni[0] + uni[3];
+  const int n_items = a.identity ? a.n : min(n_second + uni[4], a.n);
+  // slots: contributions go to per-slot stores (needs the stored short list and
+  // its reverse map); otherwise FP64 atomics into the fallback buffer
+  const bool slots_ok = uni[1] == 0;
+  // the stored short list holds every atom that can be inside a cutoff while no
+  // atom has moved more than half the list margin since the build (uniform)
+  const bool use_short = __int_as_float(uni[2]) <= a.dlim2;
+  const bool slots = !a.atomic_mode && use_short && slots_ok;
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.flags[FLAG_EXTRA] = slots ? 0 : 1;
+  __shared__ typename SumT<T>::type tsum[7][BLOCK];
+  const bool want_acc = a.acc != nullptr;
+  if (want_acc)
+    for (int q = 0; q < 7; ++q) sum_zero(tsum[q][threadIdx.x]);
+  const ItemEnv<T> v{srec, sfilt, snear, ns, n_first, n_second, n_items, slots, use_short, want_acc,
+                     &tsum[0][threadIdx.x]};
+  const bool any = force_items<T, NS, ZC, MODE, BATCH, CS, EV>(a, v, blockIdx.x * BLOCK + threadIdx.x,
+                                                               gridDim.x * BLOCK);
   if (EV >= 1 && want_acc && __syncthreads_or(any)) block_reduce_sums(&tsum[0][threadIdx.x], a.acc);
   if (a.left_reset) {
     // every block read the leftover count (uni[0]) before taking its ticket

@@ -65,7 +65,7 @@ struct LaneEnv {
 
 // One atom by W lanes. Every lane of the warp calls it; `have`: the group has
 // an atom. Returns whether the atom is left (more bonds than lanes).
-template <int NS, int W, int MODE, bool BATCH, int EV>
+template <int NS, int W, int MODE, int BATCH, int EV>
 __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneEnv& v, int i, bool have) {
   const int lane = threadIdx.x & 31, q = lane & (W - 1), gb = lane & ~(W - 1);
   const int ns = NS > 0 ? NS : v.ns;
