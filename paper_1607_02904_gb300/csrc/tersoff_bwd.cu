@@ -609,6 +609,14 @@ __global__ void __launch_bounds__(BwdBlock<T>::size) k_tersoff_bwd(const __grid_
     if (sgrad[q] != 0.0) atomicAdd(&a.grad[q], sgrad[q]);
 }
 
+}  // namespace bwd
+}  // namespace tgb
+
+#include "tersoff_bwd64.cuh"
+
+namespace tgb {
+namespace bwd {
+
 // ------------------------------------------------------------------ Hessian-vector product
 // The position derivative of the force term: d/dx [sum_a gF_a . F_a] =
 // -sum_i d/dx D_w E_i, D_w E_i the derivative of E_i along the bond
@@ -1066,6 +1074,20 @@ BwdArgs<T> make_args(Ctx* c, const T* raw, const double* gE, const double* gF, d
   return a;
 }
 
+// The FP64 path with one or two species: eight lanes per atom.
+template <int NT>
+int launch_lanes64(Ctx* c, const BwdArgs<double>& a, cudaStream_t s) {
+  void (*k)(BwdArgs<double>, int) = c->n_sys > 0 ? k_bwd_lanes64<NT, true> : k_bwd_lanes64<NT, false>;
+  constexpr size_t dyn = l64_dyn<NT>();
+  TGB_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  const int full = (c->n + L64_BLOCK / L64_W - 1) / (L64_BLOCK / L64_W);
+  const int resident = (c->n_sm > 0 ? c->n_sm : 152) * 3;  // one wave of looping blocks
+  k<<<full < resident ? full : resident, L64_BLOCK, dyn, s>>>(a, c->fx_cut_j ? 1 : 0);
+  c->launches++;
+  TGB_CUDA(c, cudaGetLastError());
+  return TERSOFF_OK;
+}
+
 template <class T>
 int launch_t(Ctx* c, const T* raw, const double* gE, const double* gF, double* grad,
              cudaStream_t s) {
@@ -1084,15 +1106,21 @@ int launch_t(Ctx* c, const T* raw, const double* gE, const double* gF, double* g
     c->fine_valid = true;
   }
   if (c->n > 0) a.fine = c->d_fine;
+  if constexpr (sizeof(T) == 8) {
+    if (c->n > 0 && c->ns == 1) return launch_lanes64<1>(c, a, s);
+    if (c->n > 0 && c->ns == 2) return launch_lanes64<2>(c, a, s);
+  }
   constexpr size_t dyn = slot_bytes<T>();
   const int grid = (c->n + B - 1) / B;
   if (grid > 0) {
     // two species on the mixed path: register accumulators (NS = 2)
-    const bool two = c->ns == 2 && sizeof(T) == sizeof(float);
-    void (*k)(BwdArgs<T>) = c->n_sys > 0 ? (two ? k_tersoff_bwd<T, 2, true> : k_tersoff_bwd<T, 0, true>)
-                            : c->ns == 1 ? k_tersoff_bwd<T, 1, false>
-                            : two        ? k_tersoff_bwd<T, 2, false>
-                                         : k_tersoff_bwd<T, 0, false>;
+    void (*k)(BwdArgs<T>) = c->n_sys > 0 ? k_tersoff_bwd<T, 0, true> : k_tersoff_bwd<T, 0, false>;
+    if constexpr (sizeof(T) == 4) {
+      if (c->ns == 2)
+        k = c->n_sys > 0 ? k_tersoff_bwd<T, 2, true> : k_tersoff_bwd<T, 2, false>;
+      else if (c->ns == 1 && c->n_sys == 0)
+        k = k_tersoff_bwd<T, 1, false>;
+    }
     // static parameter tables plus the bond slots exceed the default 48 KB
     TGB_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     k<<<grid, B, dyn, s>>>(a);
