@@ -165,6 +165,8 @@ int ensure_nbr(Ctx* c) {
     TGB_CUDA(c, cudaMalloc(&c->d_contrib, bytes ? bytes : 16));
     TGB_CUDA(c, cudaMalloc(&c->d_own, e4 * (c->n ? c->n : 1)));
     TGB_CUDA(c, cudaMemset(c->d_own, 0, e4 * (c->n ? c->n : 1)));
+    // new slots hold anything: every entry may be nonzero
+    if (c->n > 0) TGB_CUDA(c, cudaMemset(c->d_kmask, 0xff, sizeof(unsigned long long) * c->n));
     c->contrib_alloc = bytes;
     c->contrib_prec = c->precision;
   }
@@ -930,15 +932,15 @@ static int md_rerun(Ctx* c, double* x, double* v, double* f, double dt, int nste
   return TERSOFF_OK;
 }
 
-// The steps of a small system by the resident kernel (md_resident.cu): one
-// launch per stretch between rebuilds. With displacement-triggered rebuilds
-// the host reads where a launch ended; a fixed period needs no reading.
-constexpr int RESIDENT_STEPS = 4096;
-static int md_resident(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
-                       double* rows, double* thermo, cudaStream_t s) {
+// Steps of a small system by the resident kernel (md_resident.cu): one launch
+// per stretch between rebuilds. With displacement-triggered rebuilds the host
+// reads where a launch ended (not under capture); a fixed period needs no
+// reading and can be captured.
+constexpr int RESIDENT_STEPS = 4096;  // a bound on the time one launch takes
+static int enqueue_resident(Ctx* c, double* x, double* v, double* f, double dt, int nsteps,
+                            int rebuild_every, double* rows, double* thermo, cudaStream_t s) {
   int st;
   const bool on_skin = rebuild_every == TERSOFF_REBUILD_ON_SKIN;
-  const int ssb0 = c->steps_since_build;
   if (rows) TGB_CUDA(c, cudaMemsetAsync(rows, 0, sizeof(double) * tgb::ACC_LEN * (size_t)nsteps, s));
   int done = 0;         // the next launch's first step
   bool resume = false;  // ... has been drifted
@@ -953,7 +955,6 @@ static int md_resident(Ctx* c, double* x, double* v, double* f, double dt, int n
         tail = true;
       }
     }
-    // (a bound on the time one launch takes)
     const bool more = s1 - done > RESIDENT_STEPS;
     if (more) {
       s1 = done + RESIDENT_STEPS;
@@ -982,7 +983,14 @@ static int md_resident(Ctx* c, double* x, double* v, double* f, double dt, int n
   double* ke_row = rows ? rows + tgb::ACC_LEN * (size_t)(nsteps - 1) + 7 * tgb::ACC_STRIDE : nullptr;
   if ((st = tgb::launch_final_kick(c, v, f, ke_row, s))) return st;
   if (thermo && (st = tgb::launch_thermo_rows(c, rows, nsteps, tgb::MVV2E, thermo, s))) return st;
-  if ((st = tgb::read_flags(c, s))) return st;
+  return TERSOFF_OK;
+}
+
+// After a call's steps and the reading of their flags: takes the last build's
+// counts; reruns the call when a build inside overflowed, restores its start
+// when a bounded wait gave up.
+static int md_finish(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
+                     double* rows, double* thermo, int ssb0, cudaStream_t s) {
   if (c->h_flags[tgb::FLAG_MD_TIMEOUT]) {
     const size_t m = 3 * (size_t)c->n;
     TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
@@ -993,7 +1001,7 @@ static int md_resident(Ctx* c, double* x, double* v, double* f, double dt, int n
     return tgb::fail(c, TERSOFF_E_TIMEOUT, "a wait between MD steps gave up (state restored; rebuild the list)");
   }
   if (c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE])
-    return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, on_skin ? c->steps_since_build : ssb0, s);
+    return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
   c->max_cnt = c->h_flags[tgb::FLAG_OVERFLOW];
   c->max_short = c->h_flags[tgb::FLAG_SHORT_MAX];
   for (int b = 0; b < 3; ++b) c->nbucket[b] = c->h_flags[tgb::flag_bucket(b)];
@@ -1057,16 +1065,24 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     if ((st = tgb::dev_alloc(c, &c->d_snap, 3 * m))) return st;
     c->snap_alloc = 3 * m;
   }
-  if (!c->timing && tgb::resident_fits(c, rows != nullptr))
-    return md_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, s);
   const int ssb0 = on_skin ? -1 : c->steps_since_build;
+  // small systems: the resident kernel. Calls that hold whole rebuild periods
+  // replay it and its rebuilds as a graph (calls of another length meet the
+  // period at another phase each time, and the graph would be captured anew);
+  // displacement-triggered rebuilds are the host's decision
+  const bool resident = !c->timing && tgb::resident_fits(c, rows != nullptr);
+  if (resident && !(rebuild_every > 0 && nsteps % rebuild_every == 0)) {
+    if ((st = enqueue_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, s))) return st;
+    if ((st = tgb::read_flags(c, s))) return st;
+    return md_finish(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
+  }
   auto& G = c->graph;
   const bool same = G.exec && G.gen == c->gen && G.x == x && G.v == v && G.f == f &&
                     G.snap == c->d_snap &&
                     G.thermo == thermo && G.dt == dt && G.nsteps == nsteps &&
                     G.rebuild_every == rebuild_every && G.ssb0 == ssb0 &&
                     G.precision == c->precision && G.timing == c->timing &&
-                    G.decisions == tgb::bucket_decisions(c) &&
+                    G.decisions == tgb::bucket_decisions(c) && G.resident == resident &&
                     std::memcmp(&G.coef, &c->coef, sizeof(tgb::Coef)) == 0;
   if (!same) {
     tgb::drop_graph(c);
@@ -1078,7 +1094,8 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     const long long l0 = c->launches;
     c->capturing = true;
     c->timer_sink = &G.timers;
-    st = enqueue_md(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, false, cs, c->d_snap);
+    st = resident ? enqueue_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, cs)
+                  : enqueue_md(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, false, cs, c->d_snap);
     c->capturing = false;
     c->timer_sink = nullptr;
     cudaError_t ce = cudaStreamEndCapture(cs, &graph);
@@ -1109,6 +1126,7 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     G.timing = c->timing;
     G.gen = c->gen;
     G.decisions = tgb::bucket_decisions(c);
+    G.resident = resident;
     G.kernels = c->launches - l0;
     c->launches = l0;
     c->last_rebuilds = 0;  // nothing ran yet
@@ -1136,14 +1154,7 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     c->last_rebuilds = c->h_flags[tgb::FLAG_NREBUILD];
     c->launches += (long long)c->last_rebuilds * G.body_kernels;
   }
-  const bool bad = c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE];
-  if (!bad) {
-    c->max_cnt = c->h_flags[tgb::FLAG_OVERFLOW];
-    c->max_short = c->h_flags[tgb::FLAG_SHORT_MAX];
-    for (int b = 0; b < 3; ++b) c->nbucket[b] = c->h_flags[tgb::flag_bucket(b)];
-    return TERSOFF_OK;
-  }
-  return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
+  return md_finish(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
 }
 
 int tersoff_md_step(tersoff_ctx* p, double* x, double* v, double* f, int n, const double* mass,

@@ -137,7 +137,12 @@ void launch_lanes(Ctx* c, const FwdArgs<double>& a, long long items, cudaStream_
   constexpr int ATOMS = LBLOCK / W;
   const long long full = ((long long)c->n + ATOMS - 1) / ATOMS;
   long long grid = (items + ATOMS - 1) / ATOMS + (items < c->n ? 8 : 0);
-  if (c->opt_waves > 0 && c->n_sm > 0) grid = std::min(grid, (long long)c->opt_waves * c->n_sm * 5);
+  const long long wave = (long long)(c->n_sm > 0 ? c->n_sm : 152) * 6;  // resident blocks (the launch bound)
+  if (c->opt_waves > 0) grid = std::min(grid, c->opt_waves * wave);
+  // with energy or virial sums one wave of looping blocks: each block adds its
+  // totals to the accumulator once, and every such addition rounds at the
+  // total's last place
+  if (a.acc != nullptr) grid = std::min(grid, wave);
   grid = std::max(1ll, std::min(grid, full));
   const int evm = ev_mode<double, BATCH>(a);
   if constexpr (W == 4 && !BATCH) {

@@ -291,6 +291,7 @@ struct Ctx {
     bool timing = false;
     long long gen = -1;
     int decisions = -1;     // bucket_decisions() at capture
+    bool resident = false;  // the steps run in the resident kernel
     long long kernels = 0;  // kernel launches inside the graph, conditional bodies excluded
     long long body_kernels = 0;  // kernel launches of one conditional rebuild
   } graph;

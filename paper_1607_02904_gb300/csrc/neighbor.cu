@@ -250,8 +250,10 @@ __device__ int block_excl_scan(int v, int* total) {
   return res;
 }
 
+// fill (grids of one tile; else null): receives the prefixes too, which are
+// then final
 __global__ void k_scan_tiles(int* __restrict__ in, int m, int* __restrict__ out,
-                             int* __restrict__ tile_sums) {
+                             int* __restrict__ tile_sums, int* __restrict__ fill) {
   pdl_wait();
   int base = blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
   int v[SCAN_ITEMS];
@@ -266,7 +268,10 @@ __global__ void k_scan_tiles(int* __restrict__ in, int m, int* __restrict__ out,
   int total;
   int pre = block_excl_scan(s, &total);
   for (int q = 0; q < SCAN_ITEMS; ++q) {
-    if (base + q < m) out[base + q] = pre;
+    if (base + q < m) {
+      out[base + q] = pre;
+      if (fill) fill[base + q] = pre;
+    }
     pre += v[q];
   }
   if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
@@ -532,6 +537,148 @@ __global__ void __launch_bounds__(128) k_neigh(
   }
 }
 
+// The same lists by one warp per atom, for small systems: a thread per atom
+// walks 27 cells one after the other, some 30 us of dependent loads however
+// few atoms there are. Here lane q takes stencil cell q (in the order of the
+// loops above), tests its candidates (at most 32 at a time) and keeps the hits
+// as bits; prefix sums over the lanes give each cell's place in the lists, so
+// that entries stand in the same order.
+constexpr int NW_BLOCK = 512;  // 16 atoms
+template <bool BATCH>
+__global__ void __launch_bounds__(NW_BLOCK) k_neigh_warp(
+    int n, const double* __restrict__ x, const float4* __restrict__ pos32,
+    const int* __restrict__ cell_of, const int* __restrict__ cell_start,
+    const float4* __restrict__ posc, const __grid_constant__ GridDev g1,
+    const GridDev* __restrict__ geo,
+    const int* __restrict__ atom_sys, double rc2, float lo2, float hi2, int cap,
+    uint32_t* __restrict__ nbr, int* __restrict__ cnt, const __grid_constant__ Radii lim,
+    const __grid_constant__ Radii core, int ns,
+    uint32_t* __restrict__ shortl, int* __restrict__ zcnt, int* __restrict__ bucket,
+    uint8_t* __restrict__ zwa, int* __restrict__ flags) {
+  pdl_wait();
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int i = blockIdx.x * (NW_BLOCK / 32) + wid;
+  const bool active = i < n;
+  int count = 0, z = 0, zw = 0;
+  if (active) {  // warp-uniform
+    const GridDev& g = grid_of<BATCH>(g1, geo, atom_sys, i);
+    const float4 pi = pos32[i];
+    const int ti = __float_as_int(pi.w);
+    const int ci = cell_of[i] - g.cell_base;
+    int s0 = 0, s1 = 0;
+    float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+    uint32_t code = 0;
+    if (lane < 27) {
+      const int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = lane / 9 - 1;
+      int ax = ci % g.nc[0] + ox, ay = (ci / g.nc[0]) % g.nc[1] + oy, az = ci / (g.nc[0] * g.nc[1]) + oz;
+      ax += (ax < 0) ? g.nc[0] : 0;
+      ax -= (ax >= g.nc[0]) ? g.nc[0] : 0;
+      ay += (ay < 0) ? g.nc[1] : 0;
+      ay -= (ay >= g.nc[1]) ? g.nc[1] : 0;
+      az += (az < 0) ? g.nc[2] : 0;
+      az -= (az >= g.nc[2]) ? g.nc[2] : 0;
+      const int c = g.cell_base + (az * g.nc[1] + ay) * g.nc[0] + ax;
+      s0 = cell_start[c];
+      s1 = cell_start[c + 1];
+      sx = ox * g.hf[0];
+      sy = oy * g.hf[1];
+      sz = oz * g.hf[2];
+      code = ((uint32_t)(ox + 1) << 26) | ((uint32_t)(oy + 1) << 28) | ((uint32_t)(oz + 1) << 30);
+    }
+    // cells of more than 32 atoms in rounds: a round takes every lane's next 32
+    // (the order over lanes then holds within a round only, so cells this full
+    // are walked one after the other instead)
+    int most = s1 - s0;
+    for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(FULL, most, o));
+    const int turns = most <= 32 ? 1 : 27;
+    for (int turn = 0; turn < turns; ++turn) {
+      const bool my_turn = turns == 1 || turn == lane;
+      int left = my_turn ? s1 - s0 : 0, at = s0;
+      while (__any_sync(FULL, left > 0)) {
+        const int m = left < 32 ? left : 32;
+        uint32_t in_m = 0, sh_m = 0;
+        for (int k = 0; k < m; ++k) {
+          const float4 pj = posc[at + k];
+          const int jt = __float_as_int(pj.w);
+          const int j = jt >> 2, tj = jt & 3;
+          const float dx = (pj.x - pi.x) + sx;
+          const float dy = (pj.y - pi.y) + sy;
+          const float dz = (pj.z - pi.z) + sz;
+          const float r2 = dx * dx + dy * dy + dz * dz;
+          bool in = r2 < lo2;
+          if (r2 >= lo2 && r2 <= hi2) in = exact_member(x, i, j, g, rc2, dx, dy, dz);
+          in = in && j != i;
+          if (in) {
+            in_m |= 1u << k;
+            if (r2 <= lim.r2[ti * ns + tj]) {
+              sh_m |= 1u << k;
+              zw += r2 <= core.r2[ti * ns + tj] ? 1 : 0;
+            }
+          }
+        }
+        // both prefix sums in one word (at most 32 x 32 entries a round)
+        const int mine = __popc(in_m) | (__popc(sh_m) << 16);
+        int incl = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(FULL, incl, o);
+          if (lane >= o) incl += t;
+        }
+        const int total = __shfl_sync(FULL, incl, 31);
+        int pn = count + ((incl - mine) & 0xffff), ps = z + ((incl - mine) >> 16);
+        while (in_m) {
+          const int k = __ffs(in_m) - 1;
+          in_m &= in_m - 1u;
+          const uint32_t e = (uint32_t)(__float_as_int(posc[at + k].w) >> 2) | code;
+          if (pn < cap) nbr[(size_t)pn * n + i] = e;
+          ++pn;
+          if ((sh_m >> k) & 1u) {
+            if (ps < cap) shortl[(size_t)ps * n + i] = e;
+            ++ps;
+          }
+        }
+        count += total & 0xffff;
+        z += total >> 16;
+        at += m;
+        left -= m;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) zw += __shfl_xor_sync(FULL, zw, o);
+    if (lane == 0) {
+      cnt[i] = count;
+      zcnt[i] = z;
+      zwa[i] = (uint8_t)(zw < 63 ? zw : 63);
+    }
+  }
+  __shared__ int s_max[2], s_ovf, s_cnt[3], s_base[3];
+  if (threadIdx.x == 0) {
+    s_max[0] = s_max[1] = s_ovf = 0;
+    s_cnt[0] = s_cnt[1] = s_cnt[2] = 0;
+  }
+  __syncthreads();
+  const int b = zw <= 4 ? 0 : (zw <= 8 ? 1 : 2);
+  int rank = 0;
+  if (active && lane == 0) {
+    atomicMax(&s_max[0], count);
+    atomicMax(&s_max[1], z);
+    if (count > cap) s_ovf = 1;
+    rank = atomicAdd(&s_cnt[b], 1);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (s_max[0] > 0) atomicMax(&flags[FLAG_OVERFLOW], s_max[0]);
+    if (s_max[1] > 0) atomicMax(&flags[FLAG_SHORT_MAX], s_max[1]);
+    if (s_ovf) atomicOr(&flags[FLAG_OVF_ANY], 1);
+  }
+  if (threadIdx.x < 3) s_base[threadIdx.x] = s_cnt[threadIdx.x] ? atomicAdd(&flags[flag_bucket(threadIdx.x)], s_cnt[threadIdx.x]) : 0;
+  __syncthreads();
+  if (active && lane == 0) bucket[(size_t)b * n + s_base[b] + rank] = i;
+}
+// Up to this many atoms a warp takes each. MD steps with a rebuild every ten,
+// per rebuild: 58 -> 27 us at 216 atoms, 65 -> 41 at 13,824; at 32,000 the
+// thread per atom is 12 us faster, and its stores stay coalesced from there on.
+constexpr int NEIGH_WARP_MAX = 16384;
+
 // Reverse slots: for each short-list entry (j -> i), the slot of j in i's
 // short list (255 if absent), used to gather forces without atomics.
 // The first RU entries of j's list, and the first RU entries of each of those
@@ -728,15 +875,19 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
   }
   const int m = (int)ncell + 1;
   const int ntiles = (m + SCAN_TILE - 1) / SCAN_TILE;
-  TGB_CUDA(c, launch_pdl(k_scan_tiles, ntiles, SCAN_BLOCK, 0, s, c->d_cell_count, m, c->d_cell_start, c->d_scan_tmp));
+  TGB_CUDA(c, launch_pdl(k_scan_tiles, ntiles, SCAN_BLOCK, 0, s, c->d_cell_count, m, c->d_cell_start, c->d_scan_tmp,
+                         ntiles == 1 ? c->d_cell_fill : (int*)nullptr));
+  c->launches++;
   const int scanned = ntiles > SCAN_SUM_TILES ? 1 : 0;
   if (scanned) {
     TGB_CUDA(c, launch_pdl(k_scan_sums, 1, SCAN_BLOCK, 0, s, c->d_scan_tmp, ntiles));
     c->launches++;
   }
-  TGB_CUDA(c, launch_pdl(k_scan_add, (m + SCAN_ADD_BLOCK - 1) / SCAN_ADD_BLOCK, SCAN_ADD_BLOCK, 0, s,
-                         c->d_cell_start, m, c->d_scan_tmp, scanned, c->d_cell_fill));
-  c->launches += 2;
+  if (ntiles > 1) {
+    TGB_CUDA(c, launch_pdl(k_scan_add, (m + SCAN_ADD_BLOCK - 1) / SCAN_ADD_BLOCK, SCAN_ADD_BLOCK, 0, s,
+                           c->d_cell_start, m, c->d_scan_tmp, scanned, c->d_cell_fill));
+    c->launches++;
+  }
   if (n > 0) {
     TGB_CUDA(c, launch_pdl(k_scatter, nb, B, 0, s, n, c->d_cell_of, c->d_cell_fill, c->d_cell_atoms));
     TGB_CUDA(c, launch_pdl(k_cell_sort, (int)((ncell + 255) / 256), 256, 0, s, (int)ncell, c->d_cell_start,
@@ -761,7 +912,12 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
       core.r2[a * c->ns + b] = (float)(rf * rf);
     }
   if (n > 0) {
-    if (batch)
+    if (n <= NEIGH_WARP_MAX)
+      TGB_CUDA(c, launch_pdl(batch ? k_neigh_warp<true> : k_neigh_warp<false>, (n + NW_BLOCK / 32 - 1) / (NW_BLOCK / 32), NW_BLOCK, 0, s,
+          n, x, c->d_pos32, c->d_cell_of, c->d_cell_start, c->d_posc, g, batch ? c->d_geo : (const GridDev*)nullptr,
+          batch ? c->d_atom_sys : (const int*)nullptr, rc2, lo2, hi2, c->cap, c->d_nbr, c->d_cnt, lim, core, c->ns, c->d_short,
+          c->d_zcnt, c->d_bucket, c->d_zw, c->d_flags));
+    else if (batch)
       TGB_CUDA(c, launch_pdl(k_neigh<true, false>, (n + 127) / 128, 128, 0, s,
           n, x, c->d_pos32, c->d_cell_of, c->d_cell_start, c->d_posc, g, c->d_geo,
           c->d_atom_sys, rc2, lo2, hi2, c->cap, c->d_nbr, c->d_cnt, lim, core, c->ns, c->d_short,
