@@ -15,8 +15,8 @@ template <> inline const float* rec_host<float>(Ctx* c) { return c->h_rec32.data
 template <> inline const double* rec_host<double>(Ctx* c) { return c->h_rec64.data(); }
 
 // Atoms with more than 8 bonds inside the cutoffs (bucket 2), when they are
-// over 0.5% of the atoms (e.g. SiC): the slot-cached wide kernel, on the
-// launch's stream after the main launch. A grid of a few waves loops over the
+// over 0.5% of the atoms (e.g. SiC): the slot-cached wide kernel,
+// beside the main launch (see launch_buckets). A grid of a few waves loops over the
 // bucket (its size lives on the device).
 template <class T, int NS, bool BATCH = false>
 void launch_wide(Ctx* c, const FwdArgs<T>& a, cudaStream_t s) {
@@ -178,12 +178,23 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
   const int dec = bucket_decisions(c);
   const bool split1 = (dec & 1) != 0;
   const bool fork = split1 && c->side != nullptr;
-  cudaStream_t s2 = s;
+  const bool wide = (dec & 2) != 0;
+  // The wide launch runs next to the others, and starts first: it is one wave of
+  // few warps, each a long serial chain (332 us of an evaluation of 2,097,152 SiC
+  // atoms when it followed the main launch). Evaluation 1,211 -> 1,134 us; a
+  // first evaluation of 197,432 atoms with its list build 613 -> 566 us.
+  const bool fork2 = wide && c->side != nullptr && !lanes;
+  cudaStream_t s2 = s, s3 = s;
+  if (fork || fork2) cudaEventRecord(c->ev_fork, s);
+  if (fork2) {
+    cudaStreamWaitEvent(c->side2, c->ev_fork, 0);
+    s3 = c->side2;
+  }
   if (fork) {
-    cudaEventRecord(c->ev_fork, s);
     cudaStreamWaitEvent(c->side, c->ev_fork, 0);
     s2 = c->side;
   }
+  if (wide && !lanes) launch_wide<T, NS, BATCH>(c, a, s3);
   if (split1) {
     FwdArgs<T> b1 = a;
     b1.order = c->d_bucket + 1 * (size_t)c->n;
@@ -197,7 +208,6 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
     if (!lanes) launch_t<T, NS, 8, BATCH>(c, b1, force_grid(c, 8, ev_mode<T, BATCH>(a)), s2);
   }
   // bucket 0, then bucket 1 (unless split off), then bucket 2 (general path)
-  const bool wide = (dec & 2) != 0;
   FwdArgs<T> b0 = a;
   b0.order = c->d_bucket;
   b0.n_items = c->d_flags + flag_bucket(0);
@@ -225,9 +235,10 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
         }
       }
     }
-    if (!lanes) {
-      launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
-      if (wide) launch_wide<T, NS, BATCH>(c, a, s);
+    if (!lanes) launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
+    if (fork2) {
+      cudaEventRecord(c->ev_join2, c->side2);
+      cudaStreamWaitEvent(s, c->ev_join2, 0);
     }
   }
   if (fork) {

@@ -164,10 +164,11 @@ struct Ctx {
   bool fx_cut_j = false;          // f_C(r_ik) does not depend on j
   std::vector<double> h_rec64;    // host copies
   std::vector<float> h_rec32;
-  cudaStream_t side = nullptr;    // side stream for small force launches
+  cudaStream_t side = nullptr;    // side streams for the force launches of the
+  cudaStream_t side2 = nullptr;   // smaller buckets
   cudaStream_t cap_stream = nullptr;  // stream used to capture MD graphs
   cudaStream_t body_stream = nullptr; // captures the body of a conditional rebuild
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
   float* d_filt32 = nullptr;      // (ti,tj) filter radius^2
   float* d_near32 = nullptr;      // (ti,tj): squared (smallest outer cutoff - 2e-3 A); bonds
                                   // beyond it get their exact length residual (float path)
