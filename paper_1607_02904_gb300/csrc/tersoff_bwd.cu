@@ -1074,6 +1074,13 @@ BwdArgs<T> make_args(Ctx* c, const T* raw, const double* gE, const double* gF, d
   return a;
 }
 
+// One crystal of one species on the FP64 path: a thread per atom keeps the one
+// record's sums in registers, and from here on fills the chip by itself. Si, us
+// with eight lanes / a thread per atom: 4,096 atoms 86 / 154 (lambda3 103 / 163),
+// 16,384 195 / 169 (238 / 175), 512,000 4,979 / 3,000. Two species stay with the
+// lanes at every size (SiC 4,096 atoms 172 / 2,462, 512,000 6,402 / 11,077).
+constexpr int BWD64_ONE_MAX = 10000;
+
 // The FP64 path with one or two species: eight lanes per atom.
 template <int NT>
 int launch_lanes64(Ctx* c, const BwdArgs<double>& a, cudaStream_t s) {
@@ -1107,20 +1114,18 @@ int launch_t(Ctx* c, const T* raw, const double* gE, const double* gF, double* g
   }
   if (c->n > 0) a.fine = c->d_fine;
   if constexpr (sizeof(T) == 8) {
-    if (c->n > 0 && c->ns == 1) return launch_lanes64<1>(c, a, s);
+    if (c->n > 0 && c->ns == 1 && (c->n_sys > 0 || c->n <= BWD64_ONE_MAX)) return launch_lanes64<1>(c, a, s);
     if (c->n > 0 && c->ns == 2) return launch_lanes64<2>(c, a, s);
   }
   constexpr size_t dyn = slot_bytes<T>();
   const int grid = (c->n + B - 1) / B;
   if (grid > 0) {
-    // two species on the mixed path: register accumulators (NS = 2)
+    // one species, and two on the mixed path: register accumulators (NS = 1, 2)
     void (*k)(BwdArgs<T>) = c->n_sys > 0 ? k_tersoff_bwd<T, 0, true> : k_tersoff_bwd<T, 0, false>;
     if constexpr (sizeof(T) == 4) {
-      if (c->ns == 2)
-        k = c->n_sys > 0 ? k_tersoff_bwd<T, 2, true> : k_tersoff_bwd<T, 2, false>;
-      else if (c->ns == 1 && c->n_sys == 0)
-        k = k_tersoff_bwd<T, 1, false>;
+      if (c->ns == 2) k = c->n_sys > 0 ? k_tersoff_bwd<T, 2, true> : k_tersoff_bwd<T, 2, false>;
     }
+    if (c->ns == 1 && c->n_sys == 0) k = k_tersoff_bwd<T, 1, false>;
     // static parameter tables plus the bond slots exceed the default 48 KB
     TGB_CUDA(c, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
     k<<<grid, B, dyn, s>>>(a);
