@@ -407,8 +407,9 @@ int tersoff_set_scatter(tersoff_ctx* ctx, int mode);
  * as a CUDA graph and replays it on later calls with the same arguments and
  * context state; the state is snapshotted before each replay and, if a
  * rebuild inside it exceeded the list capacity, restored and the steps rerun
- * with host-checked rebuilds. With enable == 0 every step is launched
- * directly. */
+ * with host-checked rebuilds. Small systems on the mixed path run the steps
+ * between rebuilds inside one resident kernel instead, with the same results.
+ * With enable == 0 every step is launched directly. */
 int tersoff_set_graphs(tersoff_ctx* ctx, int enable);
 
 /* Number of kernel launches this context has enqueued since creation (host
