@@ -65,11 +65,9 @@ TGB_FX_TABLE uint64_t kExp2[64] = {
 };
 
 // per i: c 2^53 with c the smallest integer >= 1024 / (1 + i/64), and
-// -log2(c / 1024) with 57 fraction bits
-struct alignas(16) LogEntry {
-  uint64_t c, l;
-};
-TGB_FX_TABLE uint64_t kLog2[128] = {
+// -log2(c / 1024) with 57 fraction bits; load_log takes a pair by one 16-byte
+// load, which its address has to be a multiple of
+alignas(16) TGB_FX_TABLE uint64_t kLog2[128] = {
     0x8000000000000000ull, 0x0000000000000000ull, 0x7e20000000000000ull, 0x000ae67673c5254full,
     0x7c20000000000000ull, 0x0016b50e297afcceull, 0x7a60000000000000ull, 0x0021320bef2e08f8ull,
     0x7880000000000000ull, 0x002c99c4d80ce2adull, 0x76c0000000000000ull, 0x003768205f24a728ull,
