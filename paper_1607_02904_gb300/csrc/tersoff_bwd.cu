@@ -29,6 +29,7 @@
 // path); every gradient sum is accumulated in double.
 #include <cstring>
 
+#include "gather.cuh"
 #include "tersoff_fwd.cuh"
 
 namespace tgb {
@@ -206,10 +207,13 @@ __device__ __forceinline__ Bo<T> bond_ad(T zeta, T be, T n) {
 }
 
 // ------------------------------------------------------------------ accumulation
-// Per-thread sums are kept in T (one atom's terms: a few dozen per field) and
-// summed over the warp in T; the warp totals go to the block and global sums
-// in double. On the mixed path this keeps the FP64 pipe out of the loops (a
-// depth-5 float tree adds ~3e-7 relative error to a warp's total).
+// Per-thread sums are kept in T (one atom's terms: a few dozen per field). Over
+// the warp floats are summed as pairs (sum and rounding errors), double plainly;
+// the warp totals go to the block and global sums in double. So the float
+// rounding of a gradient is that of its atoms' own terms, and which atoms meet
+// in a warp (their order comes from atomics) changes nothing above double
+// rounding; a plain float tree moved the gradient by 1e-9 to 1e-7 of its norm
+// from one list build to the next. The FP64 pipe stays out of the loops.
 // NS == 1: one record. NS == 2 (mixed path): the 4 records (ti, *, *) of the
 // thread's centre species, summed once per centre species. Otherwise:
 // per-block shared accumulators with shared-memory atomics.
@@ -222,6 +226,47 @@ __host__ __device__ constexpr int triplet_field(int k) {
          : k == 4 ? TERSOFF_P_D
          : k == 5 ? TERSOFF_P_H
                   : TERSOFF_P_LAMBDA3;
+}
+
+// Warp sums of the C floats get(0) ... get(C - 1) of each lane (C a power of two
+// up to 32): lanes exchange halves of what they hold, so that every lane ends
+// with one sum, then the lanes that hold the same one add theirs. Each addition's
+// rounding error is recovered exactly (TwoSum) and carried along. The totals leave
+// from C lanes at once; one lane adding all 80 of two species in turn had been a
+// tenth of the adjoint (a fitting pass over 256 cells 1,310 -> 1,175 us).
+// out(k, total) runs in one lane per k.
+template <int C, class Get, class Out>
+__device__ __forceinline__ void warp_sums(Get get, Out out) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  float s[C], e[C];
+#pragma unroll
+  for (int k = 0; k < C; ++k) {
+    s[k] = get(k);
+    e[k] = 0.0f;
+  }
+  int mine = 0, o = 16;
+#pragma unroll
+  for (int n = C / 2; n >= 1; n >>= 1, o >>= 1) {
+    const bool hi = (lane & o) != 0;
+    mine += hi ? n : 0;
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      const float rs = __shfl_xor_sync(FULL, hi ? s[k] : s[k + n], o);
+      float re = 0.0f;
+      if (n < C / 2) re = __shfl_xor_sync(FULL, hi ? e[k] : e[k + n], o);
+      s[k] = hi ? s[k + n] : s[k];
+      e[k] = __fadd_rn(hi ? e[k + n] : e[k], re);
+      two_sum_acc(s[k], e[k], rs);
+    }
+  }
+#pragma unroll
+  for (; o > 0; o >>= 1) {
+    const float rs = __shfl_xor_sync(FULL, s[0], o), re = __shfl_xor_sync(FULL, e[0], o);
+    e[0] = __fadd_rn(e[0], re);
+    two_sum_acc(s[0], e[0], rs);
+  }
+  if ((lane & (32 / C - 1)) == 0) out(mine, to_f64(s[0]) + to_f64(e[0]));
 }
 
 template <int NS, class T> struct Acc;
@@ -238,11 +283,19 @@ template <class T> struct Acc<1, T> {
     for (int k = 0; k < 7; ++k) v[triplet_field(k)] += x[k];
   }
   __device__ __forceinline__ void flush(double* sh, int) {
+    if constexpr (sizeof(T) == 4) {
+      // (v[0], m, holds 0: nothing adds to it)
+      warp_sums<16>([&](int k) { return k < NP ? v[k < NP ? k : 0] : 0.0f; },
+                    [&](int k, double t) {
+                      if (t != 0.0) atomicAdd(&sh[k], t);
+                    });
+    } else {
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      T s = v[q];
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if ((threadIdx.x & 31) == 0 && s != T(0)) atomicAdd(&sh[q], to_f64(s));
+      for (int q = 0; q < NP; ++q) {
+        T s = v[q];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0 && s != T(0)) atomicAdd(&sh[q], to_f64(s));
+      }
     }
   }
 };
@@ -285,28 +338,27 @@ template <class T> struct Acc<2, T> {
     if (tj == 0) v[0][f] += x;
     else v[3][f] += x;
   }
-  // fields a record position can receive: m never; A, lambda1, B, lambda2,
-  // beta and n only at the pair records 0 and 3
-  static __device__ __forceinline__ constexpr bool used(int r, int f) {
-    return f != TERSOFF_P_M &&
-           (r == 0 || r == 3 || f == TERSOFF_P_GAMMA || f == TERSOFF_P_LAMBDA3 ||
-            f == TERSOFF_P_C || f == TERSOFF_P_D || f == TERSOFF_P_H || f == TERSOFF_P_R ||
-            f == TERSOFF_P_D_CUT);
+  // the sums that a record position can receive, as r NP + field: m never; A,
+  // lambda1, B, lambda2, beta and n only at the pair records 0 and 3
+  static constexpr int PAIR = NP - 1, SUMS = 2 * PAIR + 2 * 7;
+  static __device__ __forceinline__ constexpr int place(int k) {
+    return k < PAIR           ? k + 1
+           : k < PAIR + 7     ? NP + triplet_field(k - PAIR)
+           : k < PAIR + 2 * 7 ? 2 * NP + triplet_field(k - PAIR - 7)
+                              : 3 * NP + k - (PAIR + 2 * 7) + 1;
   }
   // all lanes; lanes without an atom hold zeros (ti 0)
   __device__ __forceinline__ void flush(double* sh, int ti) {
+    static_assert(sizeof(T) == 4 && TERSOFF_P_M == 0 && SUMS == 40, "the mixed path's sums, in groups of 32 and 8");
 #pragma unroll
-    for (int tt = 0; tt < 2; ++tt)
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int q = 0; q < NP; ++q) {
-          if (!used(r, q)) continue;
-          T s = ti == tt ? v[r][q] : T(0);
-          for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-          if ((threadIdx.x & 31) == 0 && s != T(0))
-            atomicAdd(&sh[(4 * tt + r) * NP + q], to_f64(s));
-        }
+    for (int tt = 0; tt < 2; ++tt) {
+      auto get = [&](int k) { return ti == tt ? v[place(k) / NP][place(k) % NP] : 0.0f; };
+      auto out = [&](int k, double t) {
+        if (t != 0.0) atomicAdd(&sh[4 * tt * NP + place(k)], t);
+      };
+      warp_sums<32>(get, out);
+      warp_sums<8>([&](int k) { return get(32 + k); }, [&](int k, double t) { out(32 + k, t); });
+    }
   }
 };
 template <class T> struct Acc<0, T> {
@@ -1101,8 +1153,7 @@ int launch_t(Ctx* c, const T* raw, const double* gE, const double* gF, double* g
   BwdArgs<T> a = make_args<T>(c, raw, gE, gF, grad, s);
   constexpr int B = BwdBlock<T>::size;
   // atoms by bond count, sorted once per list (the placement order within a
-  // count comes from atomics: sorting again would change the summation order
-  // between calls on the same list); blocks of 256 cover the 64 bins
+  // count comes from atomics); blocks of 256 cover the 64 bins
   if (c->n > 0 && !c->fine_valid) {
     const int nb = (c->n + 255) / 256;
     TGB_CUDA(c, cudaMemsetAsync(c->d_zbins, 0, sizeof(int) * 64, s));
