@@ -230,9 +230,12 @@ TGB_FX int64_t log2_fixed(Mant a) {
   return (int64_t)((uint64_t)(int64_t)a.e << 57) + (int64_t)l + (int64_t)p;
 }
 
-// y0 (1 + E), y0 with 31 and E with 62 fraction bits (|E| < 2^-20): 63 bits
+// y0 (1 + E), y0 with 31 and E with 62 fraction bits: 63 bits. |E| < 2^-20, where
+// E shifted by 21 still fits its word: the approximations are good to 2^-23 (what
+// the PTX instructions state) and see their argument cut to 24 bits, 2^-22
+// together. The terms of third order left out are below 2^-60.
 TGB_FX uint64_t refine(uint32_t y0, int64_t E) {
-  return ((uint64_t)y0 << 32) + (uint64_t)(mul32s(y0, (int64_t)((uint64_t)E << 22)) >> 20);
+  return ((uint64_t)y0 << 32) + (uint64_t)(mul32s(y0, (int64_t)((uint64_t)E << 21)) >> 19);
 }
 TGB_FX float inside(float y) { return fminf(fmaxf(y, 0.5f), 0.99999994f); }
 // 1 / a

@@ -1,7 +1,11 @@
 """What the integer functions' callers and loads rely on beyond their values
 (csrc/fxmath.cuh), compiled for the host."""
+import math
 import os
+import random
 import subprocess
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1607_02904_gb300", "csrc")
 
@@ -16,3 +20,37 @@ def test_logarithm_table_is_declared_for_its_16_byte_loads(tmp_path):
     # the declaration's alignment, not where a linker happened to put the table
     out = run(tmp_path, '#include "fxmath.cuh"\n#include <cstdio>\nint main() { printf("%zu", __alignof__(tgb::fx::kLog2)); }')
     assert int(out) % 16 == 0
+
+
+FUNCTIONS = r"""
+#include "fxmath.cuh"
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+int main(int argc, char** argv) {
+  namespace fx = tgb::fx;
+  fx::host_jitter() = (float)atof(HOST_JITTER);
+  char fn[16];
+  double a;
+  while (scanf("%15s %la", fn, &a) == 2) printf("%a\n", CALL);
+}
+"""
+
+
+def evaluate(tmp_path, call, values, jitter=0.0):
+    body = FUNCTIONS.replace("HOST_JITTER", f'"{jitter}"').replace("CALL", call)
+    out = run(tmp_path, body, "".join(f"f {float(v).hex()}\n" for v in values))
+    return [float.fromhex(r) for r in out.split()]
+
+
+@pytest.mark.parametrize("jitter", [6e-7, -6e-7])
+def test_reciprocals_up_to_the_stated_error_of_their_first_approximation(tmp_path, jitter):
+    # 6e-7 and the cut argument's 2^-23 and a float rounding: 0.86 x 2^-20
+    mpmath = pytest.importorskip("mpmath")
+    mpmath.mp.dps = 50
+    r = random.Random(21)
+    v = [10 ** r.uniform(-30, 30) for _ in range(4000)] + [1.0, 2.0, 4.0, 3.9999999999999996, 1.9999999999999998]
+    for call, want in (("fx::rcp(a)", lambda t: 1 / t), ("fx::rsqrt(a)", lambda t: 1 / mpmath.sqrt(t))):
+        for a, got in zip(v, evaluate(tmp_path, call, v, jitter)):
+            w = want(mpmath.mpf(a))
+            assert abs(mpmath.mpf(got) - w) <= 0.625 * mpmath.mpf(2) ** (mpmath.frexp(w)[1] - 53), (call, a)
