@@ -14,8 +14,9 @@
 // TOMS 15 (1989) 144 and 16 (1990) 378, in base 2 and fixed point); the
 // reciprocal and the reciprocal square root refine the hardware's float
 // approximation by one step of second order. Every function's relative error
-// is below 2^-56 before its one rounding to double (the logarithm's absolute
-// error below 2^-55). Arguments outside a function's range (zero, subnormal,
+// is below 2^-56 before its one rounding to double (the fixed-point logarithm's
+// absolute error below 2^-55); the reciprocal and the square root of doubles are
+// rounded correctly, as the operations that they stand for. Arguments outside a function's range (zero, subnormal,
 // infinite, NaN, or too large for the fixed-point formats) take the CUDA
 // functions or the FP64 formulas.
 //
@@ -262,14 +263,30 @@ TGB_FX Mant rsqrt(Mant a) {
 }
 
 // ---------------------------------------------------------------- on doubles
+// 1 / x, correctly rounded: the mantissas' quotient lies within 2^-6 of n or n + 1
+// units, n its cut approximation, so that the sign of 2^106 - X (2 n + 1), X the
+// mantissa of x as an integer, says which is nearer (its low 64 bits hold it; it
+// is never 0)
 TGB_FX_CALL double rcp(double x) {
-  if (!normal(x)) return 1.0 / x;
-  const double y = pack(rcp(unpack(x)));
-  return from_bits(bits_of(y) | (bits_of(x) & 0x8000000000000000ull));
+  const Mant a = unpack(x);
+  if (!normal(x) || a.e > 1021) return 1.0 / x;
+  const Mant r = rcp(a);
+  uint64_t n = r.m >> 11;
+  n += (int64_t)((a.m >> 11) * (2 * n + 1)) < 0 ? 1 : 0;
+  return from_bits((((uint64_t)(uint32_t)(r.e + 1022) << 52) + n) | (bits_of(x) & 0x8000000000000000ull));
 }
 TGB_FX_CALL double rsqrt(double x) {
   if (!(normal(x) && x > 0.0)) return 1.0 / ::sqrt(x);
   return pack(rsqrt(unpack(x)));
+}
+// sqrt(x), correctly rounded (in the same way: by the sign of 4 x - (2 n + 1)^2 in
+// units of n squared)
+TGB_FX_CALL double sqrt(double x) {
+  if (!(normal(x) && x > 0.0)) return ::sqrt(x);
+  const Mant a = unpack(x), s = mul(a, rsqrt(a));
+  uint64_t n = s.m >> 11;
+  n += (int64_t)(((a.m >> 11) << (54 + a.e - 2 * s.e)) - (2 * n + 1) * (2 * n + 1)) > 0 ? 1 : 0;
+  return from_bits(((uint64_t)(uint32_t)(s.e + 1022) << 52) + n);
 }
 // x log2(e) with 57 fraction bits, |x| < 32
 TGB_FX int64_t log2e_times(double x) {

@@ -78,7 +78,7 @@ template <> struct BM<double> {
   static __device__ __forceinline__ void scpi(double x, double* s, double* c) {
     fx::sincospi(x, s, c);
   }
-  static __device__ __forceinline__ double sq(double x) { return x * fx::rsqrt(x); }
+  static __device__ __forceinline__ double sq(double x) { return fx::sqrt(x); }
   static __device__ __forceinline__ double rcp(double x) { return fx::rcp(x); }
   static __device__ __forceinline__ double inv(double x) { return fx::rcp(x); }
 };

@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(L64_BLOCK, 3) k_bwd_lanes64(const __grid_const
       const double x = fx::from_fixed(dx, g.fix64), y = fx::from_fixed(dy, g.fix64), z = fx::from_fixed(dz, g.fix64);
       const double r2 = x * x + y * y + z * z;
       const double ir = fx::rsqrt(r2);
-      b.r = r2 * ir;
+      b.r = fx::sqrt(r2);
       b.ux = x * ir;
       b.uy = y * ir;
       b.uz = z * ir;

@@ -54,3 +54,19 @@ def test_reciprocals_up_to_the_stated_error_of_their_first_approximation(tmp_pat
         for a, got in zip(v, evaluate(tmp_path, call, v, jitter)):
             w = want(mpmath.mpf(a))
             assert abs(mpmath.mpf(got) - w) <= 0.625 * mpmath.mpf(2) ** (mpmath.frexp(w)[1] - 53), (call, a)
+
+
+def test_reciprocal_and_square_root_are_correctly_rounded(tmp_path):
+    # the adjoint's double divisions and square roots, against the host's IEEE ones
+    r = random.Random(22)
+    v = [math.ldexp(1 + r.getrandbits(52) * 2.0 ** -52, r.randrange(-1022, 1024)) for _ in range(60000)]
+    v += [math.ldexp(m, e) for e in (-1022, -1, 0, 1, 2, 500, 1020, 1021, 1022, 1023)
+          for m in (1.0, 1 + 2.0 ** -52, 2 - 2.0 ** -52, 1.5, 1 + 2.0 ** -26, 1.9999999)]
+    v += [5e-324, 2.0 ** -1023, math.inf, 0.0]
+    v += [float(k * k) for k in range(1, 2000)] + [3.0 * 2.0 ** -1024]
+    for jitter in (0.0, 1.1e-7, -1.1e-7):
+        w = v + [-a for a in v]
+        for a, got in zip(w, evaluate(tmp_path, "fx::rcp(a)", w, jitter)):
+            assert got == (1.0 / a if a else math.copysign(math.inf, a)), a
+        for a, got in zip(v, evaluate(tmp_path, "fx::sqrt(a)", v, jitter)):
+            assert got == math.sqrt(a), a
