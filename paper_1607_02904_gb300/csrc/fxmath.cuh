@@ -301,7 +301,8 @@ TGB_FX_CALL double exp(double x) {
 }
 TGB_FX_CALL double log(double x) {
   const int e = exponent(x);
-  if (!(x > 0.0 && e >= -60 && e <= 60)) return ::log(x);
+  // between 1/2 and 2 the fixed point's absolute error is not a relative one
+  if (!(x > 0.0 && e >= -60 && e <= 60) || e == 0 || e == -1) return ::log(x);
   const int64_t v = log2_fixed(unpack(x));
   const uint64_t a = (uint64_t)(v < 0 ? -v : v);
   const int z = clz64(a);

@@ -70,3 +70,16 @@ def test_reciprocal_and_square_root_are_correctly_rounded(tmp_path):
             assert got == (1.0 / a if a else math.copysign(math.inf, a)), a
         for a, got in zip(v, evaluate(tmp_path, "fx::sqrt(a)", v, jitter)):
             assert got == math.sqrt(a), a
+
+
+def test_logarithm_is_good_to_an_ulp_near_one_too(tmp_path):
+    # an ulp is what CUDA's log states; away from 1 the fixed-point logarithm's 2^-55
+    # is a quarter of an ulp of log(2), and the product and the rounding add 0.7
+    mpmath = pytest.importorskip("mpmath")
+    mpmath.mp.dps = 50
+    r = random.Random(23)
+    v = [1 + s * 2.0 ** r.uniform(-50, -1.01) for _ in range(3000) for s in (1, -1)]
+    v += [r.uniform(0.4, 2.6) for _ in range(3000)] + [0.5, 2.0, 0.49999999999999994, 1.9999999999999998, 4.0, 1.0]
+    for a, got in zip(v, evaluate(tmp_path, "fx::log(a)", v)):
+        w = mpmath.log(mpmath.mpf(a))
+        assert got == 0 if not w else abs(mpmath.mpf(got) - w) <= mpmath.mpf(2) ** (mpmath.frexp(w)[1] - 53), a
