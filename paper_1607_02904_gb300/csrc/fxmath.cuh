@@ -360,6 +360,15 @@ TGB_FX_CALL void sincospi(double x, double* s, double* c) {
   *s = swap ? cv : sv;
   *c = swap ? sv : cv;
 }
+// v a for a logarithm's magnitude v (57 fraction bits) and -30 <= a.e <= 5; false
+// from lim (at most 62) on, where the product would leave the format
+TGB_FX bool times(uint64_t v, Mant a, int lim, int64_t& z) {
+  const uint64_t p = mulhi(v, a.m);  // 56 - a.e fraction bits
+  const int up = a.e + 1;
+  const uint64_t q = up < 0 ? p >> -up : p;
+  z = (int64_t)(q << (up > 0 ? up : 0));
+  return q < ((uint64_t)lim << 57) >> (up > 0 ? up : 0);
+}
 // b = (1 + (beta zeta)^n)^(-1/(2n)) and db/dzeta = -b u / (2 (1 + u) zeta) with
 // u = (beta zeta)^n, for zeta > 0; false when an argument is outside the
 // formats (the caller then takes the FP64 formulas)
@@ -369,18 +378,16 @@ TGB_FX_CALL bool bond(double zeta, double beta, double n, double ninv2, double* 
   if (!(bz > 0.0 && n > 0.0 && normal(zeta)) || ebz < -60 || ebz > 60 || en < -30 || en > 5 || ei < -30 || ei > 5)
     return false;
   const int64_t lg = log2_fixed(unpack(bz));
-  const uint64_t a = mulhi((uint64_t)(lg < 0 ? -lg : lg), unpack(n).m);  // |n lg| 2^(56 - en)
-  if (a >= (62ull << 56) >> (en > 0 ? en : 0)) return false;
-  const int64_t zu = (int64_t)shift(a, en + 1);
+  int64_t zu, zw;
+  if (!times((uint64_t)(lg < 0 ? -lg : lg), Mant{unpack(n).m, en}, 62, zu)) return false;
   const Mant u = exp2_fixed(lg < 0 ? -zu : zu);
   // 1 + u
   const uint64_t one = 1ull << 62;
   const uint64_t s = u.e >= 0 ? (u.m >> 1) + (one >> u.e) : one + shift(u.m >> 1, u.e);
   const int c = (int)(s >> 63);
   const Mant opu{c ? s : s << 1, (u.e > 0 ? u.e : 0) + c};
-  const uint64_t w = mulhi((uint64_t)log2_fixed(opu), unpack(ninv2).m);  // log2(1 + u)/(2n) 2^(56 - ei)
-  if (w >= (62ull << 56) >> (ei > 0 ? ei : 0)) return false;
-  const Mant bm = exp2_fixed(-(int64_t)shift(w, ei + 1));
+  if (!times((uint64_t)log2_fixed(opu), Mant{unpack(ninv2).m, ei}, 62, zw)) return false;
+  const Mant bm = exp2_fixed(-zw);
   Mant d = mul(mul(bm, u), rcp(mul(opu, unpack(zeta))));
   d.e -= 1;
   *b = pack(bm);

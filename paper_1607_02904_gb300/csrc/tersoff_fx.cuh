@@ -72,18 +72,15 @@ TGB_FX bool pair64(const FxRec& p, uint64_t rm, int re, double zeta, double* fr,
   if (!((int64_t)bits_of(zeta) > 0 && ez >= -30 && ez <= 29)) return false;
   const int64_t lz = log2_fixed(unpack(zeta));
   const int64_t lbz = lz + p.lgbeta;
-  const uint64_t a = mulhi((uint64_t)(lbz < 0 ? -lbz : lbz), p.n);  // |n log2(beta zeta)| 2^(56 - n_e)
-  if (a >= (30ull << 56) >> (p.n_e > 0 ? p.n_e : 0)) return false;
-  const int64_t au = (int64_t)shift(a, p.n_e + 1);
+  int64_t au, lb;
+  if (!times((uint64_t)(lbz < 0 ? -lbz : lbz), Mant{p.n, p.n_e}, 30, au)) return false;  // |n log2(beta zeta)|
   const int64_t zu = lbz < 0 ? -au : au;
   const Mant u = exp2_fixed(zu);
   const uint64_t one = 1ull << 62;
   const uint64_t s = u.e >= 0 ? (u.m >> 1) + (one >> u.e) : one + shift(u.m >> 1, u.e);  // 1 + u
   const int c = (int)(s >> 63);
   const int64_t l1u = log2_fixed(Mant{c ? s : s << 1, (u.e > 0 ? u.e : 0) + c});
-  const uint64_t w = mulhi((uint64_t)l1u, p.in2);  // log2(1 + u)/(2n) 2^(56 - in2_e)
-  if (w >= (16ull << 56) >> (p.in2_e > 0 ? p.in2_e : 0)) return false;
-  const int64_t lb = (int64_t)shift(w, p.in2_e + 1);
+  if (!times((uint64_t)l1u, Mant{p.in2, p.in2_e}, 16, lb)) return false;  // log2(1 + u)/(2n)
   const int64_t z1 = (int64_t)shift(mulhi(rm, p.l1), re + p.l1_e - 5);
   const int64_t z2 = (int64_t)shift(mulhi(rm, p.l2), re + p.l2_e - 5);
   const Mant ba = exp2_fixed(p.lgB - z2 - lb);

@@ -3,6 +3,7 @@
 import math
 import os
 import random
+import shutil
 import subprocess
 
 import pytest
@@ -83,3 +84,71 @@ def test_logarithm_is_good_to_an_ulp_near_one_too(tmp_path):
     for a, got in zip(v, evaluate(tmp_path, "fx::log(a)", v)):
         w = mpmath.log(mpmath.mpf(a))
         assert got == 0 if not w else abs(mpmath.mpf(got) - w) <= mpmath.mpf(2) ** (mpmath.frexp(w)[1] - 53), a
+
+
+PAIR = r"""
+#include "tersoff_fx.cuh"
+#include "params_fx.cu"
+#include <cstdio>
+using namespace tgb;
+int main() {
+  double A, B, l1, l2, beta, n, c, d, h, r, zeta;
+  while (scanf("%la %la %la %la %la %la %la %la %la %la %la", &A, &B, &l1, &l2, &beta, &n, &c, &d, &h, &r, &zeta) == 11) {
+    Ctx x;
+    x.ns = 1;
+    x.rmax_cut = 3.0;
+    x.h_rec64.assign(RSTRIDE, 0.0);
+    double* o = x.h_rec64.data();
+    o[K_A] = A, o[K_B] = B, o[K_LAM1] = l1, o[K_LAM2] = l2, o[K_BETA] = beta, o[K_N] = n;
+    o[K_GAMMA] = 1.0, o[K_H] = h, o[K_D2] = d * d, o[K_GC2D2] = c * c / (d * d), o[K_G2C2] = 2 * c * c;
+    make_fx_records(&x);
+    if (!x.fx_ok) return 1;
+    const fx::Mant m = fx::unpack(r);
+    double fr = 0, bfa = 0, dz = 0;
+    const int ok = fx::pair64(x.h_fx[0], m.m, m.e, zeta, &fr, &bfa, &dz);
+    printf("%d %a %a %a\n", ok, fr, bfa, dz);
+  }
+}
+"""
+
+
+@pytest.mark.parametrize("element", ["Si", "C"])
+def test_pair_term_takes_every_zeta_of_real_neighbourhoods(tmp_path, element):
+    """Below n = 1 too the integer formats hold the whole range (n log2(beta zeta) is
+    -21 to 0 here); the caller's FP64 formulas are for what is outside of them.
+
+    Bounds: logarithms carry 2^-55, products with n, 1/(2n) and lambda r 2^-57 each;
+    2^x turns them into relative errors (times ln 2), and one rounding adds 2^-53."""
+    mpmath = pytest.importorskip("mpmath")
+    mp, mpf = mpmath.mp, mpmath.mpf
+    mp.dps = 50
+    rec = {"Si": (1830.8, 471.18, 2.4799, 1.7322, 1.1e-6, 0.78734, 1.0039e5, 16.217, -0.59825),
+           "C": (1393.6, 346.74, 3.4879, 2.2119, 1.5724e-7, 0.72751, 3.8049e4, 4.3484, -0.57058)}[element]
+    rnd = random.Random(24)
+    calls = [rec + (rnd.uniform(1.2, 3.0), 10 ** rnd.uniform(-2, 6)) for _ in range(3000)]
+    inc = ["-I", os.path.join(os.path.dirname(os.path.dirname(CSRC)), "include"), "-I", cuda_include()]
+    (tmp_path / "t.cpp").write_text(PAIR)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, *inc, "-o", str(tmp_path / "t"), str(tmp_path / "t.cpp")], check=True)
+    text = "".join(" ".join(float(v).hex() for v in c) + "\n" for c in calls)
+    out = subprocess.run([str(tmp_path / "t")], input=text, capture_output=True, text=True, check=True).stdout
+    u53 = mpf(2) ** -53
+    rows = out.splitlines()
+    assert len(rows) == len(calls)
+    for c, row in zip(calls, rows):
+        ok, fr, bfa, dz = (float.fromhex(v) if "x" in v else float(v) for v in row.split())
+        A, B, l1, l2, beta, n, _, _, _, r, zeta = (mpf(v) for v in c)
+        assert ok, c
+        u = (beta * zeta) ** n
+        b = (1 + u) ** (-1 / (2 * n))
+        want = A * mpmath.exp(-l1 * r), -b * B * mpmath.exp(-l2 * r)
+        assert abs(mpf(fr) / want[0] - 1) <= 1.5 * u53
+        assert abs(mpf(bfa) / want[1] - 1) <= 2 * u53
+        assert abs(mpf(dz) / (-want[1] * u / (4 * (1 + u) * zeta)) - 1) <= 3 * u53
+
+
+def cuda_include():
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    d = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    if not os.path.exists(os.path.join(d, "cuda_runtime.h")):
+        pytest.skip("no CUDA headers")
+    return d
