@@ -265,7 +265,6 @@ FwdArgs<T> make_args(Ctx* c, double* f, double* acc, double* eatom, bool virial 
   if constexpr (sizeof(T) == 8) {
     if (c->fx_ok) a.fx1 = c->h_fx[0];
     a.fx = c->d_fx;
-    a.qd = c->fx_qd;
     a.cut_j = c->fx_cut_j ? 1 : 0;
   }
   a.near2 = c->d_near32;

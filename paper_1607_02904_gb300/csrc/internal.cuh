@@ -160,7 +160,6 @@ struct Ctx {
   FxRec* d_fx = nullptr;          // integer records (valid when fx_ok)
   std::vector<FxRec> h_fx;
   bool fx_ok = false;             // the table is inside the integer formats
-  int fx_qd = 0;                  // fraction bits of its bond vectors
   bool fx_cut_j = false;          // f_C(r_ik) does not depend on j
   std::vector<double> h_rec64;    // host copies
   std::vector<float> h_rec32;
@@ -398,7 +397,7 @@ inline bool comp_atom_sums(const Ctx* c) {
          c->ns == 1 && c->n_sys == 0;
 }
 
-// The integer records of a table (params_fx.cu): c->fx_ok, h_fx, fx_qd.
+// The integer records of a table (params_fx.cu): c->fx_ok, h_fx, fx_cut_j.
 void make_fx_records(Ctx* c);
 
 int fail(Ctx* c, int code, const std::string& msg);

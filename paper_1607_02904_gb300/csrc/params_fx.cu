@@ -33,7 +33,6 @@ void make_fx_records(Ctx* c) {
   const double lim = 20.0 / (1.4427 * c->rmax_cut);
   bool ok = true;
   c->fx_cut_j = true;
-  c->fx_qd = 62 - (int)std::ceil(std::log2(c->rmax_cut * 1.01));
   auto in = [&](double v, double lo, double hi) { ok = ok && v >= lo && v <= hi; };
   auto rec = [&](int i, int j, int k) { return &c->h_rec64[(size_t)((i * ns + j) * ns + k) * RSTRIDE]; };
   for (int i = 0; i < ns; ++i)

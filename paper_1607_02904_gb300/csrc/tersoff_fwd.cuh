@@ -170,7 +170,6 @@ template <class T> struct FxArgs {};
 template <> struct FxArgs<double> {
   FxRec fx1;         // the record of a one-species table
   const FxRec* fx;   // ns^3 records
-  int qd;            // fraction bits of the bond vectors
   int cut_j;         // f_C(r_ik) does not depend on j
 };
 

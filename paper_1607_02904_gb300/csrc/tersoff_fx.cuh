@@ -3,7 +3,7 @@
 // Bound: one FP64 warp instruction occupies its SM quarter's pipe for 64
 // cycles, an integer one for 1 to 2. So bond vectors, lengths, unit vectors,
 // angles, the angular function, exponentials, logarithms and the bond order
-// are formed in fixed point and mantissa-exponent pairs (fxmath.cuh, 59 bits
+// are formed in fixed point and mantissa-exponent pairs (fxmath.cuh, 57 bits
 // and more), and doubles carry only the sums of Eq. 5-7: the zeta sums, the
 // radial derivative and the force accumulation, 166 to 200 FP64 instructions
 // per atom with four bonds where the FP64 formulas take 1,012.
@@ -28,11 +28,17 @@ struct Bond64 {
   int64_t ux, uy, uz;  // unit vector, 62 fraction bits
   Mant r, ri;          // length and its reciprocal
 };
-// from the bond vector with qd fraction bits (components below 2^62)
-TGB_FX Bond64 bond64(int64_t dx, int64_t dy, int64_t dz, int qd) {
-  const uint64_t ax = (uint64_t)(dx < 0 ? -dx : dx), ay = (uint64_t)(dy < 0 ? -dy : dy),
-                 az = (uint64_t)(dz < 0 ? -dz : dz);
-  const uint64_t s = mulhi(ax, ax) + mulhi(ay, ay) + mulhi(az, az);  // 2 qd - 64 fraction bits
+// from the bond vector with q fraction bits (not 0, components below 2^62). Its
+// largest component is moved up to bit 62 first, so that the squares keep 60 bits
+// at any length.
+TGB_FX Bond64 bond64(int64_t dx, int64_t dy, int64_t dz, int q) {
+  uint64_t ax = (uint64_t)(dx < 0 ? -dx : dx), ay = (uint64_t)(dy < 0 ? -dy : dy), az = (uint64_t)(dz < 0 ? -dz : dz);
+  const int up = clz64(ax | ay | az | 1ull) - 1;
+  ax <<= up;
+  ay <<= up;
+  az <<= up;
+  const int qd = q + up;
+  const uint64_t s = (mulhi(ax, ax) + mulhi(ay, ay) + mulhi(az, az)) | 1ull;  // 2 qd - 64 fraction bits
   const int z = clz64(s);
   Bond64 b;
   const Mant r2{s << z, 127 - z - 2 * qd};

@@ -157,8 +157,7 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
   if (mine) {
     Bond<double>::fixed(a, sh, pi, e, bx, by, bz, j, tj);
     if (coarse2(a, bx, by, bz) <= v.sfilt[ti * ns + tj]) {
-      const int up = a.qd - a.fix64;
-      b = fx::bond64(bx << up, by << up, bz << up, a.qd);
+      b = fx::bond64(bx, by, bz, a.fix64);
       r = fx::pack_in(b.r);
       const double* pq = v.srec + rec_off<NS>(ns, ti, tj, tj);
       const long long rb = __double_as_longlong(r);  // positive doubles order like their bits

@@ -152,3 +152,48 @@ def cuda_include():
     if not os.path.exists(os.path.join(d, "cuda_runtime.h")):
         pytest.skip("no CUDA headers")
     return d
+
+
+BOND = r"""
+#include "tersoff_fx.cuh"
+#include <cstdio>
+int main() {
+  long long x, y, z;
+  int q;
+  while (scanf("%lld %lld %lld %d", &x, &y, &z, &q) == 4) {
+    const auto b = tgb::fx::bond64(BOND_CALL);
+    printf("%a %lld %lld %lld\n", tgb::fx::pack_in(b.r), (long long)b.ux, (long long)b.uy, (long long)b.uz);
+  }
+}
+"""
+
+
+def test_bond_lengths_keep_their_bits_for_close_pairs(tmp_path):
+    """Lengths from 1e-6 A up and every scale of positions: the square to 2^-57, its
+    root to 2^-56 (fxmath) and a rounding to double; unit vectors to 2^-56 of 1."""
+    mpmath = pytest.importorskip("mpmath")
+    mp, mpf = mpmath.mp, mpmath.mpf
+    mp.dps = 50
+    rnd = random.Random(25)
+    calls = []
+    for _ in range(4000):
+        q = rnd.choice([30, 44, 52, 57])
+        r = 10 ** rnd.uniform(-6 if q > 44 else -2, 0.6)
+        d = [rnd.gauss(0, 1) * rnd.choice([1, 1, 1e-3, 0]) for _ in range(3)]
+        n = math.sqrt(sum(v * v for v in d)) or 1.0
+        v = [int(r * c / n * 2.0 ** q) for c in d]
+        if any(v):
+            calls.append((*v, q))
+    calls += [(1, 0, 0, 52), (0, -1, 0, 52), (1, 1, 1, 52), ((1 << 62) - 1, 0, 0, 60), (1 << 61, -(1 << 61), 1 << 61, 60)]
+    inc = ["-I", os.path.join(os.path.dirname(os.path.dirname(CSRC)), "include"), "-I", cuda_include()]
+    (tmp_path / "t.cpp").write_text(BOND.replace("BOND_CALL", "x, y, z, q"))
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, *inc, "-o", str(tmp_path / "t"), str(tmp_path / "t.cpp")], check=True)
+    out = subprocess.run([str(tmp_path / "t")], input="".join("%d %d %d %d\n" % c for c in calls), capture_output=True,
+                         text=True, check=True).stdout.splitlines()
+    assert len(out) == len(calls)
+    for c, row in zip(calls, out):
+        r, *u = row.split()
+        n = mpmath.sqrt(mpf(c[0]) ** 2 + mpf(c[1]) ** 2 + mpf(c[2]) ** 2)
+        assert abs(mpf(float.fromhex(r)) * mpf(2) ** c[3] / n - 1) <= mpf(2) ** -53 + mpf(2) ** -55, c
+        for a, b in zip(c[:3], u):
+            assert abs(mpf(int(b)) / mpf(2) ** 62 - a / n) <= mpf(2) ** -56, c
