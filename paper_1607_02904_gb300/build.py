@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libtersoff_gb300.so")
-SOURCES = ["tersoff_bwd.cu", "fwd_f32.cu", "fwd_f64.cu", "fwd_f64_two.cu", "fwd_f64_any.cu", "fwd_f64_batch.cu",
+SOURCES = ["tersoff_bwd.cu", "fwd_f32.cu", "fwd_f64.cu", "fwd_f64_two.cu", "fwd_f64_any.cu", "fwd_f64_batch.cu", "fwd_f64_long.cu",
            "md_resident.cu", "fwd_f32_cs.cu", "fwd_f32_quad.cu", "api.cu", "neighbor.cu", "integrate.cu", "noalloc.cu", "peaks.cu",
            "halo.cu", "checkpoint.cu", "params_fx.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

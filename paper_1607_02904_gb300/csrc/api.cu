@@ -198,7 +198,9 @@ int setup_grid(Ctx* c, const double* box, double r_list) {
   // offsets u = x - o stay within [-8, h + 8) A between rebuilds; 2^S such
   // that (h + 8) 2^S < 2^30 keeps differences inside int32
   g.fix_shift = (int)std::floor(30.0 - std::log2(hmax + 8.0));
-  g.fix64 = fix64_of(std::fmax(box[0], std::fmax(box[1], box[2])));
+  const double lmax = std::fmax(box[0], std::fmax(box[1], box[2]));
+  g.fix64 = fix64_of(lmax, c->rmax_cut);
+  g.long64 = long64_of(lmax);
   return TERSOFF_OK;
 }
 
@@ -582,7 +584,8 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
     G.invL[a] = G.invh[a] = 1.0 / hmax;
   }
   G.fix_shift = (int)std::floor(30.0 - std::log2(hmax + 8.0));
-  G.fix64 = tgb::fix64_of(lmax);
+  G.fix64 = tgb::fix64_of(lmax, c->rmax_cut);
+  G.long64 = tgb::long64_of(lmax);
   const double scale = std::ldexp(1.0, G.fix_shift);
   for (int q = 0; q < n_sys; ++q) {
     for (int a = 0; a < 3; ++a) {

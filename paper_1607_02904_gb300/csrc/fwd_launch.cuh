@@ -121,10 +121,10 @@ bool use_quad(const Ctx* c) {
 // atom through Algorithm 2's loops, keep k_tersoff.
 inline bool use_lanes64(const Ctx* c) { return c->fx_ok && !(c->ablate & TERSOFF_ABLATE_GENERAL); }
 
-template <int NS, int W, bool BATCH, int EV>
+template <int NS, int W, bool BATCH, int EV, int LONG = 0>
 void launch_lanes_ev(Ctx* c, const FwdArgs<double>& a, int grid, cudaStream_t s) {
   const bool sym = c->sym_table;  // (false with a lambda3 term)
-  void (*k)(FwdArgs<double>) = sym ? k_lanes64<NS, W, 3, BATCH, EV> : k_lanes64<NS, W, 1, BATCH, EV>;
+  void (*k)(FwdArgs<double>) = sym ? k_lanes64<NS, W, 3, BATCH, EV, LONG> : k_lanes64<NS, W, 1, BATCH, EV, LONG>;
   const size_t dyn = lanes_dyn(sym ? 3 : 1);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
   launch_pdl(k, grid, LBLOCK, dyn, s, a);
@@ -132,7 +132,7 @@ void launch_lanes_ev(Ctx* c, const FwdArgs<double>& a, int grid, cudaStream_t s)
 }
 // items: about how many atoms the launch has (the device's counts decide; the
 // kernel loops over what its grid does not cover)
-template <int NS, int W, bool BATCH>
+template <int NS, int W, bool BATCH, int LONG>
 void launch_lanes(Ctx* c, const FwdArgs<double>& a, long long items, cudaStream_t s) {
   constexpr int ATOMS = LBLOCK / W;
   const long long full = ((long long)c->n + ATOMS - 1) / ATOMS;
@@ -145,35 +145,38 @@ void launch_lanes(Ctx* c, const FwdArgs<double>& a, long long items, cudaStream_
   if (a.acc != nullptr) grid = std::min(grid, wave);
   grid = std::max(1ll, std::min(grid, full));
   const int evm = ev_mode<double, BATCH>(a);
-  if constexpr (W == 4 && !BATCH) {
+  if constexpr (W == 4 && !BATCH && !LONG) {
     if (evm == 0) return launch_lanes_ev<NS, W, BATCH, 0>(c, a, (int)grid, s);
     if (evm == 1) return launch_lanes_ev<NS, W, BATCH, 1>(c, a, (int)grid, s);
   }
-  launch_lanes_ev<NS, W, BATCH, 2>(c, a, (int)grid, s);
+  launch_lanes_ev<NS, W, BATCH, 2, LONG>(c, a, (int)grid, s);
 }
 
-template <class T, int NS, bool BATCH = false>
+// LONG: boxes with a long edge, lanes only.
+template <class T, int NS, bool BATCH = false, int LONG = 0>
 void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
   constexpr bool D = sizeof(T) == 8;
-  const bool lanes = D && use_lanes64(c);
-  if (use_quad<T, NS, BATCH>(c)) {
-    TimedRegion tr(c, 0, s);
-    const bool ev = a.acc != nullptr || a.eatom != nullptr;
-    FwdArgs<T> aq = a;
-    aq.identity = 1;
-    launch_forward_quad(c, &aq, ev, s);
-    // the atoms it left (more than four bonds inside the cutoffs, general
-    // path): the per-thread kernel over the leftover list, one block per SM
-    // looping over it; its last block zeroes the list's count
-    FwdArgs<T> bl = a;
-    bl.order = c->d_left;
-    bl.n_items = c->d_flags + FLAG_LEFT;
-    bl.order2 = bl.order3 = nullptr;
-    bl.n_items2 = bl.n_items3 = nullptr;
-    bl.identity = 0;
-    bl.left_reset = 1;
-    launch_t<T, NS, 8, BATCH>(c, bl, c->n_sm > 0 ? c->n_sm : 152, s);
-    return;
+  const bool lanes = LONG || (D && use_lanes64(c));
+  if constexpr (!D) {
+    if (use_quad<T, NS, BATCH>(c)) {
+      TimedRegion tr(c, 0, s);
+      const bool ev = a.acc != nullptr || a.eatom != nullptr;
+      FwdArgs<T> aq = a;
+      aq.identity = 1;
+      launch_forward_quad(c, &aq, ev, s);
+      // the atoms it left (more than four bonds inside the cutoffs, general
+      // path): the per-thread kernel over the leftover list, one block per SM
+      // looping over it; its last block zeroes the list's count
+      FwdArgs<T> bl = a;
+      bl.order = c->d_left;
+      bl.n_items = c->d_flags + FLAG_LEFT;
+      bl.order2 = bl.order3 = nullptr;
+      bl.n_items2 = bl.n_items3 = nullptr;
+      bl.identity = 0;
+      bl.left_reset = 1;
+      launch_t<T, NS, 8, BATCH>(c, bl, c->n_sm > 0 ? c->n_sm : 152, s);
+      return;
+    }
   }
   const int dec = bucket_decisions(c);
   const bool split1 = (dec & 1) != 0;
@@ -194,7 +197,9 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
     cudaStreamWaitEvent(c->side, c->ev_fork, 0);
     s2 = c->side;
   }
-  if (wide && !lanes) launch_wide<T, NS, BATCH>(c, a, s3);
+  if constexpr (!LONG) {
+    if (wide && !lanes) launch_wide<T, NS, BATCH>(c, a, s3);
+  }
   if (split1) {
     FwdArgs<T> b1 = a;
     b1.order = c->d_bucket + 1 * (size_t)c->n;
@@ -203,9 +208,11 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
     b1.n_items2 = b1.n_items3 = nullptr;
     b1.identity = 0;
     if constexpr (D) {
-      if (lanes) launch_lanes<NS, 8, BATCH>(c, b1, c->nbucket[1], s2);
+      if (lanes) launch_lanes<NS, 8, BATCH, LONG>(c, b1, c->nbucket[1], s2);
     }
-    if (!lanes) launch_t<T, NS, 8, BATCH>(c, b1, force_grid(c, 8, ev_mode<T, BATCH>(a)), s2);
+    if constexpr (!LONG) {
+      if (!lanes) launch_t<T, NS, 8, BATCH>(c, b1, force_grid(c, 8, ev_mode<T, BATCH>(a)), s2);
+    }
   }
   // bucket 0, then bucket 1 (unless split off), then bucket 2 (general path)
   FwdArgs<T> b0 = a;
@@ -225,17 +232,19 @@ void launch_buckets(Ctx* c, FwdArgs<T> a, cudaStream_t s) {
         long long items = c->n;
         if (split1) items -= c->nbucket[1];
         if (wide) items -= c->nbucket[2];
-        launch_lanes<NS, 4, BATCH>(c, b0, items, s);
+        launch_lanes<NS, 4, BATCH, LONG>(c, b0, items, s);
         if (wide) {
           FwdArgs<T> b2 = a;
           b2.order = c->d_bucket + 2 * (size_t)c->n;
           b2.n_items = c->d_flags + flag_bucket(2);
           b2.identity = 0;
-          launch_lanes<NS, 16, BATCH>(c, b2, c->nbucket[2], s);
+          launch_lanes<NS, 16, BATCH, LONG>(c, b2, c->nbucket[2], s);
         }
       }
     }
-    if (!lanes) launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
+    if constexpr (!LONG) {
+      if (!lanes) launch_t<T, NS, 4, BATCH>(c, b0, force_grid(c, 4, ev_mode<T, BATCH>(a)), s);
+    }
     if (fork2) {
       cudaEventRecord(c->ev_join2, c->side2);
       cudaStreamWaitEvent(s, c->ev_join2, 0);

@@ -19,11 +19,16 @@ struct alignas(32) dpos4 {
 };
 
 // Position record of the FP64 path: the coordinates wrapped into the box, in
-// 64-bit fixed point with Grid::fix64 fraction bits (finer than a double's at
-// any coordinate from the middle of the box up, at most 2^-53 A off below),
-// and the species. Differences are exact integers, and a box edge (rounded
-// once) is added or subtracted where the minimum image asks for it: bond
-// vectors carry none of the rounding of cell origins.
+// 64-bit fixed point with Grid::fix64 fraction bits, and in w the species (low
+// 32 bits). Differences are exact integers, and a box edge (rounded once) is
+// added or subtracted where the minimum image asks for it: bond vectors carry
+// none of the rounding of cell origins.
+// The rounding, 2^-(fix64 + 1) A: up to a longest edge of 2^11 A fix64 takes all
+// the bits that differences over the box leave (62 - log2 of the edge: 2^-53 A or
+// less up to 1,024 A, 2^-52 to 2,048). Beyond, the words hold the coordinate
+// modulo 2^64 at 51 fraction bits (2^-52 A up to 2^17 A), and w the coordinate in
+// units of 2^58 of them, ten bits an axis from bit 32 on, which tell the image
+// (nearest_long); from 2^17 A on fix64 gives way to those ten bits.
 struct alignas(32) ipos4 {
   long long x, y, z, w;
 };
@@ -92,6 +97,7 @@ struct Grid {
   double invh[3]; // nc / L
   int fix_shift;  // fixed-point scale 2^fix_shift for mixed positions
   int fix64;      // scale 2^fix64 of the FP64 path's positions
+  int long64;     // their coarse words are in use
 };
 
 // MD coefficients per species: c = dt/2 * (force-to-acceleration) / m, and m
@@ -113,25 +119,37 @@ struct GridDev {
   float hf[3];
 };
 
-// Box edges for the FP64 path: in fixed point (scale 2^fix64), and 1 / L.
+// Box edges for the FP64 path: in fixed point (scale 2^fix64; modulo 2^64), in
+// units of 2^58 of it, and 1 / L.
+constexpr int LONG64_UNIT = 58, LONG64_EDGE = 16;  // edges from 16 units on are long
 struct Box64 {
   long long L[3];
-  double invL[3];
+  int Lc[3];
+  double edge[3], invL[3];
   float invLf[3];
 };
 inline Box64 make_box64(const double* L, int fix64) {
   Box64 b;
   for (int a = 0; a < 3; ++a) {
-    b.L[a] = llrint(ldexp(L[a], fix64));
+    const double units = ldexp(L[a], fix64 - LONG64_UNIT);
+    b.Lc[a] = units < 1024.0 ? (int)units : 1024;
+    b.L[a] = b.Lc[a] < LONG64_EDGE ? llrint(ldexp(L[a], fix64))
+                                   : (long long)((unsigned long long)b.Lc[a] << LONG64_UNIT) +
+                                         llrint(ldexp(units - b.Lc[a], LONG64_UNIT));
+    b.edge[a] = L[a];
     b.invL[a] = 1.0 / L[a];
     b.invLf[a] = (float)b.invL[a];
   }
   return b;
 }
-// A scale that leaves int64 room for differences over two boxes.
-inline int fix64_of(double lmax) {
+// The scale for a longest edge lmax and a largest cutoff rmax (bond vectors below
+// 2^60), and whether it needs the coarse words.
+inline bool long64_of(double lmax) { return lmax > 2048.0; }
+inline int fix64_of(double lmax, double rmax) {
   const int e = (int)ceil(log2(lmax));
-  return e <= 8 ? 52 : 60 - e;
+  if (!long64_of(lmax)) return 62 - e;
+  const int f = 68 - e < 51 ? 68 - e : 51, r = 60 - (int)ceil(log2(rmax));
+  return f < r ? f : r;
 }
 
 // Periodic shift units of one system of a batch: the edges of its list cells,
@@ -423,6 +441,9 @@ int launch_neighbor_export(Ctx* c, int* cnt, int* nbr, int cap, cudaStream_t s);
 // the float offsets and the displacement references; otherwise the running
 // maximum displacement since the build is updated.
 int launch_pack_positions(Ctx* c, const double* x, bool build, cudaStream_t s);
+// After any packing of positions: the FP64 path's in boxes with a long edge
+// (nothing elsewhere).
+int launch_pos_long(Ctx* c, const double* x, cudaStream_t s);
 
 // Forces (fwd_f32.cu / fwd_f64*.cu). Accumulates into f (zeroed by the caller),
 // energy and virial into acc components 0..6 (zeroed by the caller); eatom optional.
@@ -433,6 +454,9 @@ int launch_forward_f32(Ctx* c, double* f, double* acc, double* eatom, cudaStream
                        bool virial);
 int launch_forward_f64_two(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
                            bool virial);
+int launch_forward_f64_long(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
+                            bool virial);
+int launch_forward_batch_f64_long(Ctx* c, double* f, cudaStream_t s);
 int launch_forward_f64_any(Ctx* c, double* f, double* acc, double* eatom, cudaStream_t s,
                            bool virial);
 // the force launches of the TERSOFF_ABLATE_COMP_ATOM_SUMS variant (fwd_f32_cs.cu),

@@ -871,6 +871,8 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
       bp.kmask = c->d_kmask;
       TGB_CUDA(c, launch_pdl(c->precision == TERSOFF_FP64 ? k_bin_pack<true> : k_bin_pack<false>, nb, B, 0, s, n, x, g, bp, c->d_cell_of, c->d_cell_count,
                              c->d_qorg, c->d_flags));
+      const int st = launch_pos_long(c, x, s);
+      if (st) return st;
     }
   }
   const int m = (int)ncell + 1;

@@ -39,6 +39,15 @@ __device__ __forceinline__ ipos4 make_pos64(double x, double y, double z, int t,
   return ipos4{wrap64(x, q, b.L[0], b.invL[0], b.invLf[0]), wrap64(y, q, b.L[1], b.invL[1], b.invLf[1]),
                wrap64(z, q, b.L[2], b.invL[2], b.invLf[2]), t};
 }
+// axis a of a box with a long edge: where that one is long, the coordinate modulo
+// 2^64, its coarse word to w
+__device__ __forceinline__ long long wrap_long(double x, int q, const Box64& b, int a, long long& w) {
+  if (b.Lc[a] < LONG64_EDGE) return wrap64(x, q, b.L[a], b.invL[a], b.invLf[a]);
+  const double k = floor(x * b.invL[a]);
+  const int c = (int)floor(ldexp(fma(-k, b.edge[a], x), q - LONG64_UNIT));
+  w |= (long long)min(max(c, 0), 1023) << (32 + 10 * a);
+  return (long long)((unsigned long long)to_fixed(x, q) - (unsigned long long)(long long)k * (unsigned long long)b.L[a]);
+}
 // difference of two wrapped coordinates, as the minimum image (edges are at
 // least twice the list radius, so an entry's image is the nearest one)
 __device__ __forceinline__ long long nearest(long long d, long long L) {
@@ -46,6 +55,17 @@ __device__ __forceinline__ long long nearest(long long d, long long L) {
   d -= d > half ? L : 0;
   d += d < -half ? L : 0;
   return d;
+}
+// the same on an axis of Lc units: the coarse words hi and hj (at bit s) tell the
+// image and whether the atoms are far apart (beyond any cutoff, which is below 4
+// units); the difference modulo 2^64 is the rest
+__device__ __forceinline__ long long nearest_long(long long d, long long L, int Lc, int hi, int hj, int s) {
+  if (Lc < LONG64_EDGE) return nearest(d, L);
+  int dc = ((hj >> s) & 1023) - ((hi >> s) & 1023);
+  const int k = dc > (Lc >> 1) ? 1 : (dc < -(Lc >> 1) ? -1 : 0);
+  dc -= k * Lc;
+  if (dc > 8 || dc < -8) return dc > 0 ? (1ll << 61) : -(1ll << 61);
+  return (long long)((unsigned long long)d - (unsigned long long)(long long)k * (unsigned long long)L);
 }
 
 }  // namespace tgb

@@ -183,6 +183,7 @@ template <class T> struct FwdArgs : FxArgs<T> {
   const int4* posq;      // mixed: fixed-point u, type
   const ipos4* pos64;    // fp64: fixed-point position, type
   int fix64;             // its scale 2^fix64
+  int long64;            // a long box edge: coarse words (ipos4)
   int coarse64;          // bits dropped for the float filter of its differences
   float coarse_inv;      // ... and what one of the others is, in A
   Box64 box;             // (single systems)
@@ -231,6 +232,7 @@ template <class T> struct FwdArgs : FxArgs<T> {
 template <class T> void set_pos64(const Ctx* c, FwdArgs<T>& a) {
   a.pos64 = c->d_pos64;
   a.fix64 = c->grid.fix64;
+  a.long64 = c->grid.long64;
   a.box = make_box64(c->grid.L, c->grid.fix64);
   // differences of up to four list radii fit the filter's 32 bits
   int keep = 30 - (int)ceil(log2(4.0 * c->r_list));
@@ -266,17 +268,19 @@ __device__ __forceinline__ void decode(uint32_t e, int& j, int& ox, int& oy, int
 // systems) those of atom i's system, loaded once per atom. Mixed path: the
 // list cells' edges; FP64 path: the box. KIND: 0 one system, 1 a batch, 2 one
 // system whose positions change while the kernel runs (the resident MD loop):
-// their loads must not go through the read-only path.
-template <class T, int KIND> struct Shift {
+// their loads must not go through the read-only path. LONG (FP64 path): whether a
+// box edge is long, 2: as the launch says.
+template <class T, int KIND, int LONG = 2> struct Shift {
   __device__ __forceinline__ void load(const FwdArgs<T>&, int) {}
   __device__ __forceinline__ int hq(const FwdArgs<T>& a, int q) const { return a.hq[q]; }
   __device__ __forceinline__ float h(const FwdArgs<T>& a, int q) const { return a.h[q]; }
   __device__ __forceinline__ long long L(const FwdArgs<T>& a, int q) const { return a.box.L[q]; }
+  __device__ __forceinline__ int Lc(const FwdArgs<T>& a, int q) const { return a.box.Lc[q]; }
   __device__ __forceinline__ int4 posq(const FwdArgs<T>& a, int j) const {
     return KIND == 2 ? a.posq[j] : __ldg(&a.posq[j]);
   }
 };
-template <> struct Shift<float, 1> {
+template <> struct Shift<float, 1, 2> {
   int hq_[3];
   float h_[3];
   __device__ __forceinline__ void load(const FwdArgs<float>& a, int i) {
@@ -291,13 +295,16 @@ template <> struct Shift<float, 1> {
   __device__ __forceinline__ float h(const FwdArgs<float>&, int q) const { return h_[q]; }
   __device__ __forceinline__ int4 posq(const FwdArgs<float>& a, int j) const { return __ldg(&a.posq[j]); }
 };
-template <> struct Shift<double, 1> {
+template <int LONG> struct Shift<double, 1, LONG> {
   long long L_[3];
+  int sys_;
   __device__ __forceinline__ void load(const FwdArgs<double>& a, int i) {
-    const SysShift& s = a.sys[a.atom_sys[i]];
+    sys_ = a.atom_sys[i];
+    const SysShift& s = a.sys[sys_];
 #pragma unroll
     for (int q = 0; q < 3; ++q) L_[q] = s.box.L[q];
   }
+  __device__ __forceinline__ int Lc(const FwdArgs<double>& a, int q) const { return a.sys[sys_].box.Lc[q]; }
   __device__ __forceinline__ long long L(const FwdArgs<double>&, int q) const { return L_[q]; }
 };
 
@@ -322,19 +329,26 @@ template <> struct Bond<float> {
 };
 template <> struct Bond<double> {
   // the bond vector as exact integers (scale 2^fix64)
-  template <int B>
-  static __device__ __forceinline__ void fixed(const FwdArgs<double>& a, const Shift<double, B>& sh,
+  template <int B, int LONG>
+  static __device__ __forceinline__ void fixed(const FwdArgs<double>& a, const Shift<double, B, LONG>& sh,
                                                const ipos4& pi, uint32_t e, long long& dx,
                                                long long& dy, long long& dz, int& j, int& tj) {
     j = (int)(e & ENTRY_JMASK);
     const ipos4 pj = a.pos64[j];
-    dx = nearest(pj.x - pi.x, sh.L(a, 0));
-    dy = nearest(pj.y - pi.y, sh.L(a, 1));
-    dz = nearest(pj.z - pi.z, sh.L(a, 2));
+    if (LONG == 1 || (LONG == 2 && a.long64)) {
+      const int hi = (int)(pi.w >> 32), hj = (int)(pj.w >> 32);
+      dx = nearest_long(pj.x - pi.x, sh.L(a, 0), sh.Lc(a, 0), hi, hj, 0);
+      dy = nearest_long(pj.y - pi.y, sh.L(a, 1), sh.Lc(a, 1), hi, hj, 10);
+      dz = nearest_long(pj.z - pi.z, sh.L(a, 2), sh.Lc(a, 2), hi, hj, 20);
+    } else {
+      dx = nearest(pj.x - pi.x, sh.L(a, 0));
+      dy = nearest(pj.y - pi.y, sh.L(a, 1));
+      dz = nearest(pj.z - pi.z, sh.L(a, 2));
+    }
     tj = (int)pj.w;
   }
-  template <int B>
-  static __device__ __forceinline__ void vec(const FwdArgs<double>& a, const Shift<double, B>& sh,
+  template <int B, int LONG>
+  static __device__ __forceinline__ void vec(const FwdArgs<double>& a, const Shift<double, B, LONG>& sh,
                                              const ipos4& pi, uint32_t e, double& dx, double& dy,
                                              double& dz, int& j, int& tj) {
     long long ix, iy, iz;
@@ -411,8 +425,8 @@ template <> struct Exact<float> {
   }
 };
 template <> struct Exact<double> {
-  template <int B>
-  static __device__ double residual(const FwdArgs<double>&, const Shift<double, B>&, const ipos4&,
+  template <int B, int LONG>
+  static __device__ double residual(const FwdArgs<double>&, const Shift<double, B, LONG>&, const ipos4&,
                                     uint32_t, double) {
     return 0.0;
   }
@@ -430,8 +444,8 @@ template <int B>
 __device__ __forceinline__ int4 self_pos(const FwdArgs<float>& a, const Shift<float, B>& sh, int i) {
   return sh.posq(a, i);
 }
-template <int B>
-__device__ __forceinline__ ipos4 self_pos(const FwdArgs<double>& a, const Shift<double, B>&, int i) {
+template <int B, int LONG>
+__device__ __forceinline__ ipos4 self_pos(const FwdArgs<double>& a, const Shift<double, B, LONG>&, int i) {
   return a.pos64[i];
 }
 template <>
@@ -602,8 +616,8 @@ __device__ __forceinline__ int rec_off(int ns, int ti, int tj, int tk) {
 // use_mask: bit s of mask marks the entries s < 64 inside the filter radius
 // (the others cannot be in any term and are skipped before their bond vector
 // is formed).
-template <class T, int NS, bool LAM3, int BATCH>
-__device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T, BATCH>& sh,
+template <class T, int NS, bool LAM3, int BATCH, int LONG>
+__device__ __forceinline__ void general_atom(const FwdArgs<T>& a, const Shift<T, BATCH, LONG>& sh,
                                           const T* srec, int i, int ti,
                                           const uint32_t* list, int c, bool slots,
                                           bool use_mask, unsigned long long mask, T& ei,

@@ -28,6 +28,10 @@
 // the cutoffs than lanes joins a block-local list and is done by 16 lanes, one
 // with more than 16 by one thread over its list (the general path).
 //
+// LONG: boxes with an edge beyond 2,048 A (pos64.cuh), as instances for a run-time
+// species count with energy and virial: the choice of the image inside the other
+// instances cost 2.6% of ten MD steps of 512,000 atoms.
+//
 // Forces: per-slot stores into the receiving atoms' columns (gather scatter)
 // or FP64 atomics, with the kmask bookkeeping of k_tersoff.
 #pragma once
@@ -65,13 +69,13 @@ struct LaneEnv {
 
 // One atom by W lanes. Every lane of the warp calls it; `have`: the group has
 // an atom. Returns whether the atom is left (more bonds than lanes).
-template <int NS, int W, int MODE, int BATCH, int EV>
+template <int NS, int W, int MODE, int BATCH, int EV, int LONG>
 __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneEnv& v, int i, bool have) {
   const int lane = threadIdx.x & 31, q = lane & (W - 1), gb = lane & ~(W - 1);
   const int ns = NS > 0 ? NS : v.ns;
   int zl = 0, ti = 0;
   ipos4 pi{};
-  Shift<double, BATCH> sh;
+  Shift<double, BATCH, LONG> sh;
   if (have) {
     zl = a.zcnt[i];
     pi = a.pos64[i];
@@ -368,7 +372,7 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
     }
     if (v.want_acc && near) {
       v.tsum[0] += V;
-      if (EV == 2)
+      if (EV == 2 && (!LONG || a.virial))
         for (int p = 0; p < 6; ++p) v.tsum[(1 + p) * LBLOCK] += w[p];
     }
     if (a.eatom) {
@@ -385,7 +389,7 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
   return left && q == 0;
 }
 
-template <int NS, int W, int MODE, bool BATCH, int EV>
+template <int NS, int W, int MODE, bool BATCH, int EV, int LONG>
 __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ FwdArgs<double> a) {
   static_assert(EV == 2 || !BATCH, "batches need the per-atom energy and virial");
   pdl_wait();
@@ -439,7 +443,7 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
                   : item < n1  ? a.order[item]
                   : item < n2  ? a.order2[item - n1]
                                : a.order3[item - n2];
-    const bool left = lanes_atom<NS, W, MODE, BATCH, EV>(a, v, i, have);
+    const bool left = lanes_atom<NS, W, MODE, BATCH, EV, LONG>(a, v, i, have);
     if (left) over_a[atomicAdd(&over[0], 1)] = i;
     // what did not fit: 16 lanes, then a thread each (the barrier's own count,
     // the same for every thread, decides)
@@ -449,7 +453,7 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
         for (int b0 = 0; b0 < na; b0 += LBLOCK / 16) {
           const int k = b0 + threadIdx.x / 16;
           const int i2 = k < na ? over_a[k] : 0;
-          if (lanes_atom<NS, 16, MODE, BATCH, EV>(a, v, i2, k < na)) over_b[atomicAdd(&over[1], 1)] = i2;
+          if (lanes_atom<NS, 16, MODE, BATCH, EV, LONG>(a, v, i2, k < na)) over_b[atomicAdd(&over[1], 1)] = i2;
         }
         __syncthreads();
       }
@@ -459,7 +463,7 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
         const int ig = rest[threadIdx.x];
         atomicAdd(&a.flags[FLAG_FALLBACK], 1);
         if (!v.slots && !a.atomic_mode) clear_slots<double>(a, ig);
-        Shift<double, BATCH> sh;
+        Shift<double, BATCH, LONG> sh;
         sh.load(a, ig);
         const int zl = a.zcnt[ig], ti = a.types[ig];
         const bool in_short = v.use_short && zl <= a.zs_cap;
@@ -476,7 +480,8 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
           if (a.eatom) a.eatom[ig] = eg;
           if (v.want_acc) {
             v.tsum[0] += eg;
-            for (int p = 0; p < 6; ++p) v.tsum[(1 + p) * LBLOCK] += w[p];
+            if (!LONG || a.virial)
+              for (int p = 0; p < 6; ++p) v.tsum[(1 + p) * LBLOCK] += w[p];
           }
           if (BATCH)
             for (int p = 0; p < 6; ++p) a.vatom[6 * (size_t)ig + p] = w[p];
