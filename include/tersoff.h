@@ -154,7 +154,10 @@ int tersoff_neighbor_export(tersoff_ctx* ctx, int* cnt, int* nbr, int cap, void*
  * forces[N x 3], virial[6] = (xx, yy, zz, xy, xz, yz) with
  * W_ab = sum over terms of (x_a - x_i)_a F_b relative to each term's centre
  * atom i (positive = repulsive); any output may be NULL. Outputs are
- * overwritten, not accumulated. */
+ * overwritten, not accumulated. On the FP64 path (tables inside its integer
+ * formats, as all published ones are) a position that is not finite, or two
+ * atoms at one place, make energy, virial and the forces of the atoms that
+ * have them in their lists NaN. */
 int tersoff_compute(tersoff_ctx* ctx, const double* x, int n, double* energy,
                     double* forces, double* virial, void* stream);
 

@@ -180,6 +180,7 @@ TGB_FX double pack(Mant a) {
   const uint64_t b = ((uint64_t)(uint32_t)(a.e + 1022) << 52) + r;
   return a.e < -1022 ? 0.0 : from_bits(a.e > 1023 || b > 0x7ff0000000000000ull ? 0x7ff0000000000000ull : b);
 }
+TGB_FX double nan64() { return from_bits(0x7ff8000000000000ull); }
 // v 2^-q, rounded to nearest (|v| > 0 or 0)
 TGB_FX double from_fixed(int64_t v, int q) {
   const uint64_t a = (uint64_t)(v < 0 ? -v : v);

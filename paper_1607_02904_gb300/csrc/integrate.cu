@@ -27,7 +27,7 @@ __global__ void k_pos_long(const __grid_constant__ PackArgs a, const double* __r
   const Box64& b = a.sys ? a.sys[a.atom_sys[i]].box : a.box;
   const double* xi = x + 3 * (size_t)i;
   ipos4 p;
-  p.w = a.types[i];
+  p.w = word64(xi[0], xi[1], xi[2], a.types[i]);
   p.x = wrap_long(xi[0], a.fix64, b, 0, p.w);
   p.y = wrap_long(xi[1], a.fix64, b, 1, p.w);
   p.z = wrap_long(xi[2], a.fix64, b, 2, p.w);

@@ -29,9 +29,13 @@ struct alignas(32) dpos4 {
 // modulo 2^64 at 51 fraction bits (2^-52 A up to 2^17 A), and w the coordinate in
 // units of 2^58 of them, ten bits an axis from bit 32 on, which tell the image
 // (nearest_long); from 2^17 A on fix64 gives way to those ten bits.
+// Fixed point has no NaN: an atom with a coordinate that is not finite carries
+// POS64_BAD in w.
 struct alignas(32) ipos4 {
   long long x, y, z, w;
 };
+constexpr long long POS64_BAD = 1ll << 62;
+__host__ __device__ inline bool pos64_bad(const ipos4& p) { return (int)(p.w >> 32) >= (int)(POS64_BAD >> 32); }
 
 // ------------------------------------------------------------------ parameters
 // Derived parameter record, one per (ti, tj, tk), RSTRIDE values of T.

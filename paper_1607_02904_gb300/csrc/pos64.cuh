@@ -35,9 +35,15 @@ __device__ __forceinline__ long long wrap64(double x, int q, long long L, double
   X -= X >= L ? L : 0;
   return X;
 }
+__device__ __forceinline__ bool not_finite(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) == 0x7ff00000u;
+}
+__device__ __forceinline__ long long word64(double x, double y, double z, int t) {
+  return t | (not_finite(x) || not_finite(y) || not_finite(z) ? POS64_BAD : 0ll);
+}
 __device__ __forceinline__ ipos4 make_pos64(double x, double y, double z, int t, int q, const Box64& b) {
   return ipos4{wrap64(x, q, b.L[0], b.invL[0], b.invLf[0]), wrap64(y, q, b.L[1], b.invL[1], b.invLf[1]),
-               wrap64(z, q, b.L[2], b.invL[2], b.invLf[2]), t};
+               wrap64(z, q, b.L[2], b.invL[2], b.invLf[2]), word64(x, y, z, t)};
 }
 // axis a of a box with a long edge: where that one is long, the coordinate modulo
 // 2^64, its coarse word to w

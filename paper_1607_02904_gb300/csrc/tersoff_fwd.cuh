@@ -328,9 +328,11 @@ template <> struct Bond<float> {
   }
 };
 template <> struct Bond<double> {
-  // the bond vector as exact integers (scale 2^fix64)
+  // the bond vector as exact integers (scale 2^fix64). Positions that are not
+  // finite: with LONG 2 the vector lies beyond every cutoff; the others (k_lanes64)
+  // see to it themselves, returned is whether j's is one
   template <int B, int LONG>
-  static __device__ __forceinline__ void fixed(const FwdArgs<double>& a, const Shift<double, B, LONG>& sh,
+  static __device__ __forceinline__ bool fixed(const FwdArgs<double>& a, const Shift<double, B, LONG>& sh,
                                                const ipos4& pi, uint32_t e, long long& dx,
                                                long long& dy, long long& dz, int& j, int& tj) {
     j = (int)(e & ENTRY_JMASK);
@@ -346,6 +348,9 @@ template <> struct Bond<double> {
       dz = nearest(pj.z - pi.z, sh.L(a, 2));
     }
     tj = (int)pj.w;
+    // (an edge is at most 2^62 units, a cutoff at most half of it)
+    if (LONG == 2) dx = pos64_bad(pi) || pos64_bad(pj) ? 3ll << 60 : dx;
+    return pos64_bad(pj);
   }
   template <int B, int LONG>
   static __device__ __forceinline__ void vec(const FwdArgs<double>& a, const Shift<double, B, LONG>& sh,

@@ -82,6 +82,9 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
     ti = NS == 1 ? 0 : (int)pi.w;
     sh.load(a, i);
   }
+  // a position that is not finite, of the atom or of one on its list, or a
+  // neighbour at its own place: the lane has seen one
+  bool odd = have && pos64_bad(pi);
   const uint32_t* list = a.shortl;
   int c = zl;
   bool left = have && v.use_short && (zl > a.zs_cap || zl > 64);
@@ -110,7 +113,7 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
         es = list[(size_t)s * a.n + i];
         long long dx, dy, dz;
         int jj, tj;
-        Bond<double>::fixed(a, sh, pi, es, dx, dy, dz, jj, tj);
+        odd |= Bond<double>::fixed(a, sh, pi, es, dx, dy, dz, jj, tj);
         ok = coarse2(a, dx, dy, dz) <= v.sfilt[ti * ns + tj];
       }
       const unsigned m = (__ballot_sync(0xffffffffu, ok) >> gb) & ((1u << W) - 1u);
@@ -159,9 +162,10 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
   double fc = 0.0, dfc = 0.0, r = 1.0;
   bool near = false, taper = false;
   if (mine) {
-    Bond<double>::fixed(a, sh, pi, e, bx, by, bz, j, tj);
+    odd |= Bond<double>::fixed(a, sh, pi, e, bx, by, bz, j, tj);
     if (coarse2(a, bx, by, bz) <= v.sfilt[ti * ns + tj]) {
       b = fx::bond64(bx, by, bz, a.fix64);
+      odd |= b.r.e < -a.fix64 - 8;  // the zero vector's, far below one unit
       r = fx::pack_in(b.r);
       const double* pq = v.srec + rec_off<NS>(ns, ti, tj, tj);
       const long long rb = __double_as_longlong(r);  // positive doubles order like their bits
@@ -330,6 +334,11 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
     fy_ = fma(ri, gy, w * uy);
     fz_ = fma(ri, gz, w * uz);
   }
+  // such an atom's energy and all forces of its terms are NaN
+  if ((__ballot_sync(0xffffffffu, odd) >> gb) & ((1u << W) - 1u)) {
+    V = fx_ = fy_ = fz_ = fx::nan64();
+    near = true;
+  }
   // 5. stores: the lane's neighbour force, the atom's own (lane 0)
   const double ox = -group_sum<W>(fx_), oy = -group_sum<W>(fy_), oz = -group_sum<W>(fz_);
   if (mine) {
@@ -476,6 +485,21 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
         double eg = 0.0, w[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
         general_atom<double, NS, MODE == 1, BATCH>(a, sh, v.srec, ig, ti, list, c, v.slots && in_short, false, 0ull, eg, w);
         if (v.slots && in_short) a.kmask[ig] = ~0ull;  // every entry written
+        const ipos4 pg = a.pos64[ig];
+        bool odd = pos64_bad(pg);
+        for (int s = 0; s < c; ++s) {
+          long long dx, dy, dz;
+          int jj, tj;
+          odd |= Bond<double>::fixed(a, sh, pg, list[(size_t)s * a.n + ig], dx, dy, dz, jj, tj) || (dx | dy | dz) == 0;
+        }
+        if (odd) {
+          eg = fx::nan64();
+          for (int p = 0; p < 6; ++p) w[p] = eg;
+          if (v.slots && in_short)
+            store_slot<double>(a, a.own, (size_t)ig, eg, eg, eg);
+          else
+            atomic_add3(a.f, ig, eg, eg, eg);
+        }
         if (EV >= 1) {
           if (a.eatom) a.eatom[ig] = eg;
           if (v.want_acc) {
