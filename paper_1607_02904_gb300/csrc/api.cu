@@ -109,7 +109,9 @@ int dev_alloc(Ctx* c, T** p, size_t count) {
   return TERSOFF_OK;
 }
 
-int ensure_atoms(Ctx* c, int n) {
+// Buffers of n atoms. What has to start as zeros is cleared on the caller's stream
+// (its stream need not wait for the null stream).
+int ensure_atoms(Ctx* c, int n, cudaStream_t s) {
   if ((size_t)n <= c->atoms_alloc && c->d_types) return TERSOFF_OK;
   size_t m = (size_t)n;
   int st;
@@ -133,13 +135,13 @@ int ensure_atoms(Ctx* c, int n) {
   if ((st = dev_alloc(c, &c->d_bucket, 3 * m))) return st;
   if ((st = dev_alloc(c, &c->d_left, m))) return st;
   if ((st = dev_alloc(c, &c->d_extra, 3 * (m ? m : 1)))) return st;
-  TGB_CUDA(c, cudaMemset(c->d_extra, 0, sizeof(double) * 3 * (m ? m : 1)));
+  TGB_CUDA(c, cudaMemsetAsync(c->d_extra, 0, sizeof(double) * 3 * (m ? m : 1), s));
   c->atoms_alloc = m;
   c->nbr_alloc = 0;  // list storage depends on n
   return TERSOFF_OK;
 }
 
-int ensure_nbr(Ctx* c) {
+int ensure_nbr(Ctx* c, cudaStream_t s) {
   // at least 8 slots per atom: the force kernel loads up to 8 short-list
   // entries before it reads the count
   size_t need = (size_t)(c->cap > 8 ? c->cap : 8) * (size_t)c->n;
@@ -164,9 +166,9 @@ int ensure_nbr(Ctx* c) {
     c->d_contrib = c->d_own = nullptr;
     TGB_CUDA(c, cudaMalloc(&c->d_contrib, bytes ? bytes : 16));
     TGB_CUDA(c, cudaMalloc(&c->d_own, e4 * (c->n ? c->n : 1)));
-    TGB_CUDA(c, cudaMemset(c->d_own, 0, e4 * (c->n ? c->n : 1)));
+    TGB_CUDA(c, cudaMemsetAsync(c->d_own, 0, e4 * (c->n ? c->n : 1), s));
     // new slots hold anything: every entry may be nonzero
-    if (c->n > 0) TGB_CUDA(c, cudaMemset(c->d_kmask, 0xff, sizeof(unsigned long long) * c->n));
+    if (c->n > 0) TGB_CUDA(c, cudaMemsetAsync(c->d_kmask, 0xff, sizeof(unsigned long long) * c->n, s));
     c->contrib_alloc = bytes;
     c->contrib_prec = c->precision;
   }
@@ -215,7 +217,7 @@ int read_flags(Ctx* c, cudaStream_t s) {
 // overflow regrow; synchronises s once per attempt
 int build_list(Ctx* c, const double* x, cudaStream_t s) {
   for (int attempt = 0; attempt < 4; ++attempt) {
-    int st = ensure_nbr(c);
+    int st = ensure_nbr(c, s);
     if (st) return st;
     TGB_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int) * FLAG_BUILD_WORDS, s));
     TGB_CUDA(c, cudaMemsetAsync(c->d_flags + FLAG_NONFINITE, 0, sizeof(int), s));
@@ -281,14 +283,15 @@ int tersoff_create(tersoff_ctx** out, int precision) {
     delete p;
     return TERSOFF_E_CUDA;
   }
-  cudaMemset(c->d_flags, 0, sizeof(int) * tgb::FLAG_COUNT);
-  cudaMemset(c->d_acc, 0, sizeof(double) * tgb::ACC_LEN);
   if (cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
     c->n_sm = 0;
   if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
     c->cap_stream = nullptr;
   if (cudaStreamCreateWithFlags(&c->body_stream, cudaStreamNonBlocking) != cudaSuccess)
     c->body_stream = nullptr;
+  cudaMemsetAsync(c->d_flags, 0, sizeof(int) * tgb::FLAG_COUNT, c->cap_stream);
+  cudaMemsetAsync(c->d_acc, 0, sizeof(double) * tgb::ACC_LEN, c->cap_stream);
+  cudaStreamSynchronize(c->cap_stream);  // (the first call may come on any stream)
   int prio_lo = 0, prio_hi = 0;
   cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
   if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio_hi) != cudaSuccess ||
@@ -452,21 +455,18 @@ int tersoff_params(tersoff_ctx* p, int ns, const double* table) {
   if ((st = tgb::dev_alloc(c, &c->d_rec32, r32.size()))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_filt32, f32.size()))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_near32, near32.size()))) return st;
-  TGB_CUDA(c, cudaMemcpy(c->d_rec64, r64.data(), sizeof(double) * r64.size(), cudaMemcpyHostToDevice));
-  TGB_CUDA(c, cudaMemcpy(c->d_rec32, r32.data(), sizeof(float) * r32.size(), cudaMemcpyHostToDevice));
-  {
-    // raw records for the backward pass (table layout, both precisions)
-    const size_t nraw = (size_t)nrec * TERSOFF_NPARAM;
-    std::vector<float> raw32(nraw);
-    for (size_t q = 0; q < nraw; ++q) raw32[q] = (float)table[q];
-    if ((st = tgb::dev_alloc(c, &c->d_raw64, nraw))) return st;
-    if ((st = tgb::dev_alloc(c, &c->d_raw32, nraw))) return st;
-    TGB_CUDA(c, cudaMemcpy(c->d_raw64, table, sizeof(double) * nraw, cudaMemcpyHostToDevice));
-    TGB_CUDA(c, cudaMemcpy(c->d_raw32, raw32.data(), sizeof(float) * nraw, cudaMemcpyHostToDevice));
-  }
-  TGB_CUDA(c, cudaMemcpy(c->d_filt32, f32.data(), sizeof(float) * f32.size(), cudaMemcpyHostToDevice));
-  TGB_CUDA(c, cudaMemcpy(c->d_near32, near32.data(), sizeof(float) * near32.size(),
-                         cudaMemcpyHostToDevice));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_rec64, r64.data(), sizeof(double) * r64.size(), cudaMemcpyHostToDevice, c->cap_stream));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_rec32, r32.data(), sizeof(float) * r32.size(), cudaMemcpyHostToDevice, c->cap_stream));
+  // raw records for the backward pass (table layout, both precisions)
+  const size_t nraw = (size_t)nrec * TERSOFF_NPARAM;
+  std::vector<float> raw32(nraw);
+  for (size_t q = 0; q < nraw; ++q) raw32[q] = (float)table[q];
+  if ((st = tgb::dev_alloc(c, &c->d_raw64, nraw))) return st;
+  if ((st = tgb::dev_alloc(c, &c->d_raw32, nraw))) return st;
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_raw64, table, sizeof(double) * nraw, cudaMemcpyHostToDevice, c->cap_stream));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_raw32, raw32.data(), sizeof(float) * nraw, cudaMemcpyHostToDevice, c->cap_stream));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_filt32, f32.data(), sizeof(float) * f32.size(), cudaMemcpyHostToDevice, c->cap_stream));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_near32, near32.data(), sizeof(float) * near32.size(), cudaMemcpyHostToDevice, c->cap_stream));
   c->gen++;
   c->ns = ns;
   c->h_rec64 = r64;
@@ -480,8 +480,10 @@ int tersoff_params(tersoff_ctx* p, int ns, const double* table) {
   tgb::make_fx_records(c);
   if (c->fx_ok) {
     if ((st = tgb::dev_alloc(c, &c->d_fx, c->h_fx.size()))) return st;
-    TGB_CUDA(c, cudaMemcpy(c->d_fx, c->h_fx.data(), sizeof(tgb::FxRec) * c->h_fx.size(), cudaMemcpyHostToDevice));
+    TGB_CUDA(c, cudaMemcpyAsync(c->d_fx, c->h_fx.data(), sizeof(tgb::FxRec) * c->h_fx.size(), cudaMemcpyHostToDevice, c->cap_stream));
   }
+  // the table is in place whatever stream the next call comes on
+  TGB_CUDA(c, cudaStreamSynchronize(c->cap_stream));
   return TERSOFF_OK;
 }
 
@@ -507,7 +509,7 @@ int tersoff_neighbor_build(tersoff_ctx* p, const double* x, const int* types, in
   c->margin = 0.6 * (r_list - c->rmax_cut);
   c->have_list = false;
   c->gen++;
-  if ((st = tgb::ensure_atoms(c, n))) return st;
+  if ((st = tgb::ensure_atoms(c, n, s))) return st;
   if (n > 0)
     TGB_CUDA(c, cudaMemcpyAsync(c->d_types, types, sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
   // species range check on the device copy is folded into the build kernels'
@@ -604,14 +606,11 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
   if ((st = tgb::dev_alloc(c, &c->d_atom_sys, (size_t)n))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_eatom, (size_t)n))) return st;
   if ((st = tgb::dev_alloc(c, &c->d_vatom, 6 * (size_t)n))) return st;
-  TGB_CUDA(c, cudaMemcpy(c->d_geo, geo.data(), sizeof(tgb::GridDev) * n_sys,
-                         cudaMemcpyHostToDevice));
-  TGB_CUDA(c, cudaMemcpy(c->d_sys, shifts.data(), sizeof(tgb::SysShift) * n_sys,
-                         cudaMemcpyHostToDevice));
-  TGB_CUDA(c, cudaMemcpy(c->d_sys_off, sys_offsets, sizeof(int) * (n_sys + 1),
-                         cudaMemcpyHostToDevice));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_geo, geo.data(), sizeof(tgb::GridDev) * n_sys, cudaMemcpyHostToDevice, s));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_sys, shifts.data(), sizeof(tgb::SysShift) * n_sys, cudaMemcpyHostToDevice, s));
+  TGB_CUDA(c, cudaMemcpyAsync(c->d_sys_off, sys_offsets, sizeof(int) * (n_sys + 1), cudaMemcpyHostToDevice, s));
   if (n > 0)
-    TGB_CUDA(c, cudaMemcpy(c->d_atom_sys, asys.data(), sizeof(int) * n, cudaMemcpyHostToDevice));
+    TGB_CUDA(c, cudaMemcpyAsync(c->d_atom_sys, asys.data(), sizeof(int) * n, cudaMemcpyHostToDevice, s));
   c->n_sys = n_sys;
   c->ncell_batch = cells;
   c->n = n;
@@ -619,7 +618,7 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
   c->margin = 0.6 * (r_list - c->rmax_cut);
   c->have_list = false;
   c->gen++;
-  if ((st = tgb::ensure_atoms(c, n))) return st;
+  if ((st = tgb::ensure_atoms(c, n, s))) return st;
   if (n > 0) {
     TGB_CUDA(c, cudaMemcpyAsync(c->d_types, types, sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
     std::vector<int> ht(n);
@@ -668,7 +667,7 @@ int tersoff_neighbor_export(tersoff_ctx* p, int* cnt, int* nbr, int cap, void* s
 static int batch_impl(Ctx* c, const double* x, double* f, double* energies, double* virials,
                       cudaStream_t s) {
   int st;
-  if ((st = tgb::ensure_nbr(c))) return st;
+  if ((st = tgb::ensure_nbr(c, s))) return st;
   if ((st = tgb::launch_pack_positions(c, x, false, s))) return st;
   TGB_CUDA(c, cudaMemsetAsync(c->d_acc, 0, sizeof(double) * tgb::ACC_LEN, s));
   TGB_CUDA(c, cudaMemsetAsync(c->d_flags + tgb::FLAG_EXTRA_STICKY, 0, sizeof(int), s));
@@ -687,7 +686,7 @@ static int compute_impl(Ctx* c, const double* x, int n, double* energy, double* 
   if (n != c->n || (n > 0 && !x))
     return tgb::fail(c, TERSOFF_E_INVALID_ARG, "atom count differs from the neighbour build");
   double* f = forces ? forces : c->d_fbuf;
-  if ((st = tgb::ensure_nbr(c))) return st;
+  if ((st = tgb::ensure_nbr(c, s))) return st;
   if ((st = tgb::launch_pack_positions(c, x, false, s))) return st;
   TGB_CUDA(c, cudaMemsetAsync(c->d_acc, 0, sizeof(double) * tgb::ACC_LEN, s));
   TGB_CUDA(c, cudaMemsetAsync(c->d_flags + tgb::FLAG_EXTRA_STICKY, 0, sizeof(int), s));
@@ -1046,7 +1045,7 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
     c->coef.m[t] = hc[TERSOFF_MAX_SPECIES + t];
     c->coef.hmf[t] = (float)(0.5 * hc[TERSOFF_MAX_SPECIES + t]);
   }
-  if ((st = tgb::ensure_nbr(c))) return st;
+  if ((st = tgb::ensure_nbr(c, s))) return st;
   double* rows = nullptr;
   if (thermo) {
     const size_t need = tgb::ACC_LEN * (size_t)nsteps;
