@@ -415,6 +415,14 @@ int tersoff_set_scatter(tersoff_ctx* ctx, int mode);
  * With enable == 0 every step is launched directly. */
 int tersoff_set_graphs(tersoff_ctx* ctx, int enable);
 
+/* How many polls a wait between the blocks of that resident kernel takes at
+ * most: 1 to 4194304 (the default, about a second). A wait runs out when the
+ * GPU is held by other work for that long. The call then restores its start
+ * state and runs its steps by launches, with the same results as a call on a
+ * list built at its start, and so do the context's later calls until this or
+ * tersoff_set_graphs is called. */
+int tersoff_set_md_wait_limit(tersoff_ctx* ctx, int polls);
+
 /* Number of kernel launches this context has enqueued since creation (host
  * output); used to report launch counts. */
 int tersoff_launch_count(const tersoff_ctx* ctx, long long* count);

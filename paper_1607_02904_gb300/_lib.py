@@ -65,6 +65,7 @@ _SIG = {
     "tersoff_set_ablation": ([_P, _I], _I),
     "tersoff_set_timing": ([_P, _I], _I),
     "tersoff_set_graphs": ([_P, _I], _I),
+    "tersoff_set_md_wait_limit": ([_P, _I], _I),
     "tersoff_set_scatter": ([_P, _I], _I),
     "tersoff_timing": ([_P, _I, _P, _P], _I),
     "tersoff_pipe_peaks": ([_P, _P], _I),
@@ -300,6 +301,10 @@ class Context:
 
     def set_graphs(self, enable=True):
         self._check(self.lib.tersoff_set_graphs(self.h, int(bool(enable))))
+
+    def set_md_wait_limit(self, polls):
+        """Polls after which a wait inside the resident MD kernel gives up (tersoff_set_md_wait_limit)."""
+        self._check(self.lib.tersoff_set_md_wait_limit(self.h, int(polls)))
 
     def set_timing(self, enable=True):
         self._check(self.lib.tersoff_set_timing(self.h, int(bool(enable))))

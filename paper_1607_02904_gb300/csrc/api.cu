@@ -913,24 +913,31 @@ static int enqueue_md(Ctx* c, double* x, double* v, double* f, double dt,
 }
 
 // After a build inside a call's sequence overflowed (or met non-finite
-// positions): restores the call's start state from the snapshot, rebuilds with
-// a host check and runs the steps eagerly.
+// positions), or a bounded wait of the resident kernel gave up (timeout):
+// restores the call's start state from the snapshot, rebuilds with a host check
+// and runs the steps eagerly.
 static int md_rerun(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
-                    double* rows, double* thermo, int ssb0, cudaStream_t s) {
+                    double* rows, double* thermo, int ssb0, bool timeout, cudaStream_t s) {
   const size_t m = 3 * (size_t)c->n;
   const bool on_skin = rebuild_every == TERSOFF_REBUILD_ON_SKIN;
   int st;
   TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
   TGB_CUDA(c, cudaMemcpyAsync(v, c->d_snap + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
   TGB_CUDA(c, cudaMemcpyAsync(f, c->d_snap + 2 * m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-  if (c->h_flags[tgb::FLAG_NONFINITE]) {
+  if (timeout) {
+    // what blocks that went on scattered into the fallback buffer is nobody's
+    TGB_CUDA(c, cudaMemsetAsync(c->d_extra, 0, sizeof(double) * m, s));
+    c->use_resident = false;
+  } else if (c->h_flags[tgb::FLAG_NONFINITE]) {
     if (!on_skin) c->steps_since_build = ssb0;
     TGB_CUDA(c, cudaStreamSynchronize(s));
     return tgb::fail(c, TERSOFF_E_NONFINITE, "non-finite position during MD (state restored)");
+  } else {
+    c->cap = c->cap + c->cap / 2 + 4;
+    c->gen++;
   }
-  c->cap = c->cap + c->cap / 2 + 4;
-  c->gen++;
   if ((st = tgb::build_list(c, x, s))) return st;
+  if (timeout && !on_skin) c->steps_since_build = ssb0;  // the period goes on as it would have
   c->last_rebuilds = 0;
   st = enqueue_md(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, true, s);
   if (st) return st;
@@ -993,21 +1000,14 @@ static int enqueue_resident(Ctx* c, double* x, double* v, double* f, double dt, 
 }
 
 // After a call's steps and the reading of their flags: takes the last build's
-// counts; reruns the call when a build inside overflowed, restores its start
-// when a bounded wait gave up.
+// counts; reruns the call when a build inside overflowed or a bounded wait gave
+// up (the blocks were not all on the chip, or it was held by others for longer
+// than the wait: such a context takes launches from then on).
 static int md_finish(Ctx* c, double* x, double* v, double* f, double dt, int nsteps, int rebuild_every,
                      double* rows, double* thermo, int ssb0, cudaStream_t s) {
-  if (c->h_flags[tgb::FLAG_MD_TIMEOUT]) {
-    const size_t m = 3 * (size_t)c->n;
-    TGB_CUDA(c, cudaMemcpyAsync(x, c->d_snap, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    TGB_CUDA(c, cudaMemcpyAsync(v, c->d_snap + m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    TGB_CUDA(c, cudaMemcpyAsync(f, c->d_snap + 2 * m, sizeof(double) * m, cudaMemcpyDeviceToDevice, s));
-    TGB_CUDA(c, cudaStreamSynchronize(s));
-    c->have_list = false;
-    return tgb::fail(c, TERSOFF_E_TIMEOUT, "a wait between MD steps gave up (state restored; rebuild the list)");
-  }
-  if (c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE])
-    return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);
+  const bool timeout = c->h_flags[tgb::FLAG_MD_TIMEOUT] != 0;
+  if (timeout || c->h_flags[tgb::FLAG_OVF_ANY] || c->h_flags[tgb::FLAG_NONFINITE])
+    return md_rerun(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, timeout, s);
   c->max_cnt = c->h_flags[tgb::FLAG_OVERFLOW];
   c->max_short = c->h_flags[tgb::FLAG_SHORT_MAX];
   for (int b = 0; b < 3; ++b) c->nbucket[b] = c->h_flags[tgb::flag_bucket(b)];
@@ -1076,7 +1076,7 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
   // replay it and its rebuilds as a graph (calls of another length meet the
   // period at another phase each time, and the graph would be captured anew);
   // displacement-triggered rebuilds are the host's decision
-  const bool resident = !c->timing && tgb::resident_fits(c, rows != nullptr);
+  const bool resident = !c->timing && c->use_resident && tgb::resident_fits(c, rows != nullptr);
   if (resident && !(rebuild_every > 0 && nsteps % rebuild_every == 0)) {
     if ((st = enqueue_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, s))) return st;
     if ((st = tgb::read_flags(c, s))) return st;
@@ -1433,7 +1433,19 @@ int tersoff_set_graphs(tersoff_ctx* p, int enable) {
   Ctx* c = C(p);
   if (!c) return TERSOFF_E_INVALID_ARG;
   c->use_graphs = enable != 0;
+  c->use_resident = true;
   tgb::drop_graph(c);
+  return TERSOFF_OK;
+}
+
+int tersoff_set_md_wait_limit(tersoff_ctx* p, int polls) {
+  Ctx* c = C(p);
+  if (!c) return TERSOFF_E_INVALID_ARG;
+  if (polls < 1 || polls > tgb::MD_WAIT_POLLS)
+    return tgb::fail(c, TERSOFF_E_INVALID_ARG, "the wait limit must be in [1, 4194304]");
+  c->md_wait = polls;
+  c->use_resident = true;
+  c->gen++;
   return TERSOFF_OK;
 }
 

@@ -165,6 +165,9 @@ struct SysShift {
   Box64 box;
 };
 
+// Polls of the resident MD kernel's barrier: about a second.
+constexpr int MD_WAIT_POLLS = 1 << 22;
+
 // ------------------------------------------------------------------ context
 struct Ctx {
   int precision = TERSOFF_FP64;
@@ -301,6 +304,9 @@ struct Ctx {
   // MD steps as one CUDA graph per call shape (replayed while the shape and
   // the context state generation stay the same)
   bool use_graphs = true;
+  bool use_resident = true;            // small systems' steps in the resident kernel; false
+                                       // after one of its waits gave up
+  int md_wait = MD_WAIT_POLLS;         // polls after which a wait of its barrier gives up
   long long gen = 0;  // bumped by params, builds from outside MD, capacity changes
   struct MdGraph {
     cudaGraphExec_t exec = nullptr;

@@ -17,7 +17,9 @@
 // The barrier. Up to 16 blocks (2,048 atoms) form one cluster and use its
 // hardware barrier. More blocks count arrivals in global memory: the launch is
 // cooperative (all blocks are on the chip), every wait is bounded, and a wait
-// that runs out raises FLAG_MD_TIMEOUT and ends the kernel.
+// that runs out raises FLAG_MD_TIMEOUT and ends the kernel (the other blocks'
+// waits then run out too); the host restores the call's start and runs its steps
+// by launches.
 #include "step.cuh"
 #include "tersoff_fwd.cuh"
 
@@ -41,9 +43,8 @@ struct ResidentArgs {
   double* rows;  // thermo accumulation rows or null
   double* snap;  // receives the state that step 0 starts from
   int* flags;
+  int polls;  // of a wait before it gives up
 };
-
-constexpr unsigned SPIN_LIMIT = 1u << 22;  // about a second
 
 // Barrier over the blocks of the one cluster, and the same words.
 __device__ __forceinline__ void cluster_barrier(const int* flags, int* words) {
@@ -55,17 +56,17 @@ __device__ __forceinline__ void cluster_barrier(const int* flags, int* words) {
 // Barrier over the grid; then the words every block needs: the running
 // displacement and whether a short-list entry lacks its reverse. False: a wait
 // ran out.
-__device__ __forceinline__ bool grid_barrier(int* flags, unsigned target, int* words) {
+__device__ __forceinline__ bool grid_barrier(int* flags, unsigned target, int polls, int* words) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     int* bar = flags + FLAG_MD_BAR;
     atomicAdd(bar, 1);
-    unsigned spins = 0;
+    int spins = 0;
     unsigned have;
     do {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(have) : "l"(bar) : "memory");
-    } while ((int)(have - target) < 0 && ++spins < SPIN_LIMIT);
+    } while ((int)(have - target) < 0 && ++spins < polls);
     const bool ok = (int)(have - target) >= 0;
     if (!ok) atomicExch(flags + FLAG_MD_TIMEOUT, 1);
     __threadfence();
@@ -94,6 +95,9 @@ __global__ void __launch_bounds__(BLOCK, 6)
     sfilt[threadIdx.x] = a.filt2[threadIdx.x];
     snear[threadIdx.x] = a.near2[threadIdx.x];
   }
+  // a wait of an earlier launch of the call gave up: its steps will be run again
+  // (step 0's launch goes on in any case: it writes the snapshot)
+  if (!CLUSTER && r.s0 > 0 && *(const volatile int*)(r.flags + FLAG_MD_TIMEOUT)) return;
   if (threadIdx.x == 0) {
     words[0] = r.flags[FLAG_DMAX];
     words[1] = r.flags[FLAG_REV_MISS];
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(BLOCK, 6)
       target += gridDim.x;
       if (CLUSTER)
         cluster_barrier(r.flags, words);
-      else if (!grid_barrier(r.flags, target, words))
+      else if (!grid_barrier(r.flags, target, r.polls, words))
         return;
     }
     const float dmax2 = __int_as_float(words[0]);
@@ -145,7 +149,7 @@ __global__ void __launch_bounds__(BLOCK, 6)
     target += gridDim.x;
     if (CLUSTER)
       cluster_barrier(r.flags, words);
-    else if (!grid_barrier(r.flags, target, words))
+    else if (!grid_barrier(r.flags, target, r.polls, words))
       return;
   }
   if (first) r.flags[FLAG_MD_STEP] = s;
@@ -220,7 +224,7 @@ int launch_resident(Ctx* c, double* x, double* v, const double* f, double dt, in
   PackArgs pk = make_pack(c, true);
   GatherArgs ga = make_gather(c);
   Coef cf = c->coef;
-  ResidentArgs r{x, v, f, dt, s0, s1, resume, tail, on_skin, lim2, rows, snap, c->d_flags};
+  ResidentArgs r{x, v, f, dt, s0, s1, resume, tail, on_skin, lim2, rows, snap, c->d_flags, c->md_wait};
   TGB_CUDA(c, cudaMemsetAsync(c->d_flags + FLAG_MD_HALT, 0, sizeof(int) * 2 * FLAG_STRIDE, s));  // and the barrier
   void* args[] = {&a, &pk, &ga, &cf, &r};
   Config g(c, s);
