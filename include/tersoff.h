@@ -430,7 +430,10 @@ int tersoff_launch_count(const tersoff_ctx* ctx, long long* count);
 /* Kernel timing. With enable != 0 the context records a CUDA event pair on the
  * launching stream around every force-kernel launch (kind 0), every neighbour
  * build (kind 1, all of its kernels) and every integration kernel (kind 2).
- * Enabling resets the totals. */
+ * Enabling resets the totals. While it is enabled, small systems' MD steps run
+ * as launches, not in the resident kernel (tersoff_set_graphs): the times are
+ * those of the separate kernels, with the same results, and the call takes
+ * longer than without timing. */
 int tersoff_set_timing(tersoff_ctx* ctx, int enable);
 
 /* Accumulated device time in milliseconds and number of timed launches of
