@@ -122,12 +122,19 @@ bool use_quad(const Ctx* c) {
 inline bool use_lanes64(const Ctx* c) { return c->fx_ok && !(c->ablate & TERSOFF_ABLATE_GENERAL); }
 
 template <int NS, int W, bool BATCH, int EV, int LONG = 0>
-void launch_lanes_ev(Ctx* c, const FwdArgs<double>& a, int grid, cudaStream_t s) {
+void launch_lanes_ev(Ctx* c, const FwdArgs<double>& a, long long grid, cudaStream_t s) {
   const bool sym = c->sym_table;  // (false with a lambda3 term)
   void (*k)(FwdArgs<double>) = sym ? k_lanes64<NS, W, 3, BATCH, EV, LONG> : k_lanes64<NS, W, 1, BATCH, EV, LONG>;
   const size_t dyn = lanes_dyn(sym ? 3 : 1);
+  const long long wave = (long long)(c->n_sm > 0 ? c->n_sm : 152) *
+                         (sym ? lanes_blocks<NS, 3, BATCH, EV>() : lanes_blocks<NS, 1, BATCH, EV>());
+  if (c->opt_waves > 0) grid = std::min(grid, c->opt_waves * wave);
+  // with energy or virial sums one wave of looping blocks: each block adds its
+  // totals to the accumulator once, and every such addition rounds at the
+  // total's last place
+  if (a.acc != nullptr) grid = std::min(grid, wave);
   cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-  launch_pdl(k, grid, LBLOCK, dyn, s, a);
+  launch_pdl(k, (int)grid, LBLOCK, dyn, s, a);
   c->launches++;
 }
 // items: about how many atoms the launch has (the device's counts decide; the
@@ -137,19 +144,13 @@ void launch_lanes(Ctx* c, const FwdArgs<double>& a, long long items, cudaStream_
   constexpr int ATOMS = LBLOCK / W;
   const long long full = ((long long)c->n + ATOMS - 1) / ATOMS;
   long long grid = (items + ATOMS - 1) / ATOMS + (items < c->n ? 8 : 0);
-  const long long wave = (long long)(c->n_sm > 0 ? c->n_sm : 152) * 6;  // resident blocks (the launch bound)
-  if (c->opt_waves > 0) grid = std::min(grid, c->opt_waves * wave);
-  // with energy or virial sums one wave of looping blocks: each block adds its
-  // totals to the accumulator once, and every such addition rounds at the
-  // total's last place
-  if (a.acc != nullptr) grid = std::min(grid, wave);
   grid = std::max(1ll, std::min(grid, full));
   const int evm = ev_mode<double, BATCH>(a);
   if constexpr (W == 4 && !BATCH && !LONG) {
-    if (evm == 0) return launch_lanes_ev<NS, W, BATCH, 0>(c, a, (int)grid, s);
-    if (evm == 1) return launch_lanes_ev<NS, W, BATCH, 1>(c, a, (int)grid, s);
+    if (evm == 0) return launch_lanes_ev<NS, W, BATCH, 0>(c, a, grid, s);
+    if (evm == 1) return launch_lanes_ev<NS, W, BATCH, 1>(c, a, grid, s);
   }
-  launch_lanes_ev<NS, W, BATCH, 2, LONG>(c, a, (int)grid, s);
+  launch_lanes_ev<NS, W, BATCH, 2, LONG>(c, a, grid, s);
 }
 
 // LONG: boxes with a long edge, lanes only.

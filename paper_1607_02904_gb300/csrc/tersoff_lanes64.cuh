@@ -11,9 +11,13 @@
 // per atom of the same arithmetic needs 168 registers for four bonds: 11 warps
 // share an SM and 30% of the issue slots are taken (512,000 atoms, ten MD
 // steps: 4.20 ms; 4,096 atoms, one evaluation: 51 us). A lane per bond needs
-// 80 registers: 23 warps, half of the slots (3.93 ms, 33 us; the FP64 formulas
-// with integer elementary functions 5.71 ms, 52 us). Six blocks per SM: 80
-// registers; five (96) 4.09 ms, four (128) 4.62, seven (72) 4.20, eight 4.28.
+// 80 registers: 23 warps, half of the slots (3.85 ms, 32 us; the FP64 formulas
+// with integer elementary functions 5.71 ms, 52 us). That is six blocks per SM,
+// with the forces only; a launch bound of four (128 registers) 4.38 ms, five (96)
+// 4.06, seven (72) 4.02, eight (64) 4.15. Instances whose shared memory leaves
+// fewer blocks get their registers (lanes_blocks): 80 for all of them spilled 130
+// to 690 bytes (4,096 atoms, one evaluation 32.8 -> 31.6 us; an evaluation with
+// energy of 92,736 SiC atoms 259 -> 238).
 // Lists of five to eight bonds take 8 lanes and of up to sixteen 16 lanes: 24
 // fitting cells with lambda3 spend 77 and 68 us there, where a thread per atom
 // with eight bonds in registers and with bonds in shared memory took 373 and
@@ -46,6 +50,18 @@ constexpr int lanes_scratch(int W, int mode) {  // doubles per thread in dynamic
 }
 // (the block-local rest runs with 16 lanes)
 constexpr size_t lanes_dyn(int mode) { return sizeof(double) * LBLOCK * lanes_scratch(16, mode); }
+// Blocks of an instance on one SM, for its launch bound and for grids of one wave:
+// six, or what shared memory leaves (228 KB, 1 KB of it per block; the tables of
+// several species, the sums over atoms, the scratch): 5 with energy sums and one or
+// two species, 4 and 3 with lambda3, 3 and 2 for a run-time species count.
+constexpr int LANES_BLOCKS = 6;
+template <int NS, int MODE, bool BATCH, int EV> constexpr int lanes_blocks() {
+  constexpr int SNS = NS > 0 ? NS : TERSOFF_MAX_SPECIES;
+  constexpr size_t tables = NS == 1 ? 0 : (size_t)SNS * SNS * SNS * (sizeof(double) * RSTRIDE + sizeof(FxRec));
+  constexpr size_t sums = EV >= 1 && !BATCH ? sizeof(double) * (7 * LBLOCK + 8 * (LBLOCK / 32)) : 0;
+  constexpr int fit = (int)(233472 / (tables + sums + 512 + lanes_dyn(MODE) + 1024));
+  return fit < LANES_BLOCKS ? fit : LANES_BLOCKS;
+}
 
 template <class T>
 __device__ __forceinline__ T lsh(T v, int src) { return __shfl_sync(0xffffffffu, v, src); }
@@ -399,7 +415,7 @@ __device__ __forceinline__ bool lanes_atom(const FwdArgs<double>& a, const LaneE
 }
 
 template <int NS, int W, int MODE, bool BATCH, int EV, int LONG>
-__global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ FwdArgs<double> a) {
+__global__ void __launch_bounds__(LBLOCK, lanes_blocks<NS, MODE, BATCH, EV>()) k_lanes64(const __grid_constant__ FwdArgs<double> a) {
   static_assert(EV == 2 || !BATCH, "batches need the per-atom energy and virial");
   pdl_wait();
   constexpr int SNS = NS > 1 ? NS : (NS == 1 ? 1 : TERSOFF_MAX_SPECIES);
@@ -428,7 +444,7 @@ __global__ void __launch_bounds__(LBLOCK, 6) k_lanes64(const __grid_constant__ F
   }
   if (threadIdx.x < 2) over[threadIdx.x] = 0;
   LaneEnv v;
-  v.want_acc = EV >= 1 && a.acc != nullptr;
+  v.want_acc = EV >= 1 && !BATCH && a.acc != nullptr;  // (a batch's sums are per system)
   if (v.want_acc)
     for (int q = 0; q < 7; ++q) tsum[q][threadIdx.x] = 0.0;
   __syncthreads();
