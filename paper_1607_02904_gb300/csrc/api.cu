@@ -1073,11 +1073,14 @@ static int md_impl(Ctx* c, double* x, double* v, double* f, int n, const double*
   }
   const int ssb0 = on_skin ? -1 : c->steps_since_build;
   // small systems: the resident kernel. Calls that hold whole rebuild periods
-  // replay it and its rebuilds as a graph (calls of another length meet the
-  // period at another phase each time, and the graph would be captured anew);
-  // displacement-triggered rebuilds are the host's decision
-  const bool resident = !c->timing && c->use_resident && tgb::resident_fits(c, rows != nullptr);
-  if (resident && !(rebuild_every > 0 && nsteps % rebuild_every == 0)) {
+  // replay a graph (calls of another length meet the period at another phase each
+  // time, and the graph would be captured anew): of the resident kernel and the
+  // rebuilds while one cluster holds the system, else of launches, which a replay
+  // hides well enough (see RESIDENT_MAX_ATOMS); displacement-triggered rebuilds are
+  // the host's decision
+  const bool whole = rebuild_every > 0 && nsteps % rebuild_every == 0;
+  const bool resident = !c->timing && c->use_resident && tgb::resident_fits(c, whole, rows != nullptr);
+  if (resident && !whole) {
     if ((st = enqueue_resident(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, s))) return st;
     if ((st = tgb::read_flags(c, s))) return st;
     return md_finish(c, x, v, f, dt, nsteps, rebuild_every, rows, thermo, ssb0, s);

@@ -516,16 +516,26 @@ int launch_halo_pack(Ctx* c, const double* x, const int* types, const long long*
                      int* send_t, long long* send_id, int* counts, cudaStream_t s);
 
 // Resident MD kernel of small systems (md_resident.cu). resident_fits: whether
-// the context's steps run in it (rows: with thermo accumulation).
+// the context's steps run in it (whole: a call of whole rebuild periods; rows: with
+// thermo accumulation).
 // launch_resident: steps s0 .. s1 - 1 (resume: from the forces of s0, whose
 // drift ran before a rebuild; tail: then the drift of s1 before a rebuild);
 // with on_skin the kernel ends at the first step whose displacement asks for a
 // rebuild. Its end is in the FLAG_MD_* words.
-// The size limit: 512 blocks of 128 fit the chip at once, and the launches'
-// share of a step has shrunk (on-skin steps at 64,000 atoms 23.1 us resident,
-// 33.1 at 110,592 as graph nodes).
+// The size rules, us per step resident / by launches (graph replays where the call
+// allows them; Si, 1000 K):
+//   atoms                    216          2,048        4,096        32,000       65,536
+//   on skin, energies        12.5 / 22.4  14.7 / 24.1  16.9 / 24.6  20.9 / 27.8  25.1 / 31.6
+//   never                    11.8 / 19.3  13.2 / 20.2  14.5 / 20.2  18.2 / 23.0  24.5 / 28.0
+//   every 10, 25 steps       14.3 / 24.1  15.5 / 25.6  17.9 / 25.6  23.0 / 30.7  25.5 / 33.2
+//   every 10, 100 steps      12.8 / 13.2  14.0 / 15.0  16.1 / 15.0  20.9 / 19.4  23.6 / 21.6
+// A replayed graph of whole periods has no gap that the resident kernel could close,
+// and the barrier through memory costs more than its launches do: such calls stay
+// with them beyond one cluster. The others gain at every size up to the limit; at
+// 110,592 atoms on skin with energies still 33.2 / 38.5, every 10 in 100 steps
+// 29.9 / 25.2 (blocks fit the chip up to 116,736).
 constexpr int RESIDENT_MAX_ATOMS = 65536;
-bool resident_fits(Ctx* c, bool rows);
+bool resident_fits(Ctx* c, bool whole, bool rows);
 int launch_resident(Ctx* c, double* x, double* v, const double* f, double dt, int s0, int s1, bool resume, bool tail,
                     bool on_skin, float lim2, double* rows, double* snap, cudaStream_t s);
 

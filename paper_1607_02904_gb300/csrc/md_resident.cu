@@ -193,11 +193,12 @@ struct Config {
 }  // namespace
 
 // The mixed path's gathered forces in the one launch per step that small
-// systems take (no bucket on a kernel of its own), up to the size at which the
-// graph's launches are hidden.
-bool resident_fits(Ctx* c, bool rows) {
+// systems take (no bucket on a kernel of its own), up to the sizes given with
+// RESIDENT_MAX_ATOMS.
+bool resident_fits(Ctx* c, bool whole, bool rows) {
   if (c->precision != TERSOFF_MIXED || c->n_sys > 0 || c->scatter_atomic || c->ablate || c->opt_quad == 1 ||
-      c->opt_waves > 0 || c->n_sm <= 0 || c->n > RESIDENT_MAX_ATOMS || bucket_decisions(c) != 0)
+      c->opt_waves > 0 || c->n_sm <= 0 || c->n > RESIDENT_MAX_ATOMS ||
+      (whole && !one_cluster(c)) || bucket_decisions(c) != 0)
     return false;
   void* k = kernel(c, rows);
   if (one_cluster(c)) {
