@@ -4,9 +4,10 @@
 // short dependent passes (kick, drift and pack; forces); as graph nodes they
 // cost a launch each, and with displacement-triggered rebuilds a decision
 // kernel and a conditional node more: 23 us per step at 216 atoms, 28 at
-// 32,000, against 13.9 and 20.9 here (100 steps with energies at 1000 K, their
-// rebuilds included; 8.5 and 12.8 on steps without either). Here the blocks stay on the chip, one atom per thread, and a
-// barrier over the grid separates the passes. The kernel returns at the step
+// 32,000, against 13.5 and 21.1 here (100 steps with energies at 1000 K, their
+// rebuilds included; 8.5 and 12.8 on steps without either). Here the blocks stay
+// on the chip, one atom per thread, and a barrier over the grid separates the
+// passes. The kernel returns at the step
 // whose rebuild is due (a displacement beyond half the skin, or the fixed
 // period); the host enqueues the build and the rest.
 //

@@ -1128,9 +1128,9 @@ BwdArgs<T> make_args(Ctx* c, const T* raw, const double* gE, const double* gF, d
 
 // One crystal of one species on the FP64 path: a thread per atom keeps the one
 // record's sums in registers, and from here on fills the chip by itself. Si, us
-// with eight lanes / a thread per atom: 4,096 atoms 86 / 154 (lambda3 103 / 163),
+// with eight lanes / a thread per atom: 4,096 atoms 88 / 154 (lambda3 103 / 163),
 // 16,384 195 / 169 (238 / 175), 512,000 4,979 / 3,000. Two species stay with the
-// lanes at every size (SiC 4,096 atoms 172 / 2,462, 512,000 6,402 / 11,077).
+// lanes at every size (SiC 4,096 atoms 175 / 2,462, 512,000 6,575 / 11,077).
 constexpr int BWD64_ONE_MAX = 10000;
 
 // The FP64 path with one or two species: eight lanes per atom.

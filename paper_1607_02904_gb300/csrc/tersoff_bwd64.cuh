@@ -14,7 +14,7 @@
 // the columns are summed over a block once.
 // Measured: a fitting iteration of 24 cells (some 13,000 atoms, lambda3 on)
 // 3.48 -> 1.69 ms, of which the adjoint had been 2.1 ms; SiC, 4,096 atoms,
-// 2,462 -> 172 us, 512,000 atoms 11.1 -> 6.4 ms. (A large crystal of one species
+// 2,462 -> 175 us, 512,000 atoms 11.1 -> 6.6 ms. (A large crystal of one species
 // keeps a thread per atom: BWD64_ONE_MAX.)
 #pragma once
 

@@ -6,7 +6,7 @@
 // term, and, with the other bonds' dV/dzeta, the force on its neighbour
 // (second K loop). The force on the atom is the negated group sum.
 //
-// Bound: issue and latency, with the FP64 pipe 60% busy. The terms are integer
+// Bound: issue and latency, with the FP64 pipe 62% busy. The terms are integer
 // arithmetic (tersoff_fx.cuh) with some 40 FP64 instructions per lane. A thread
 // per atom of the same arithmetic needs 168 registers for four bonds: 11 warps
 // share an SM and 30% of the issue slots are taken (512,000 atoms, ten MD
