@@ -203,6 +203,7 @@ int setup_grid(Ctx* c, const double* box, double r_list) {
   const double lmax = std::fmax(box[0], std::fmax(box[1], box[2]));
   g.fix64 = fix64_of(lmax, c->rmax_cut);
   g.long64 = long64_of(lmax);
+  c->box64 = make_box64(g.L, g.fix64);
   return TERSOFF_OK;
 }
 
@@ -588,6 +589,7 @@ int tersoff_neighbor_build_batched(tersoff_ctx* p, const double* x, const int* t
   G.fix_shift = (int)std::floor(30.0 - std::log2(hmax + 8.0));
   G.fix64 = tgb::fix64_of(lmax, c->rmax_cut);
   G.long64 = tgb::long64_of(lmax);
+  c->box64 = tgb::make_box64(G.L, G.fix64);
   const double scale = std::ldexp(1.0, G.fix_shift);
   for (int q = 0; q < n_sys; ++q) {
     for (int a = 0; a < 3; ++a) {

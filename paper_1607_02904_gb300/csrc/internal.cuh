@@ -269,6 +269,8 @@ struct Ctx {
                        // (mixed path, one or two species, a single system), 0 or -1
                        // (automatic: measured slower on the benchmark) one thread per atom
   int n_sm = 0;        // multiprocessors of the device
+  Box64 box64{};       // the grid's box for the FP64 path (made with the grid: every launch
+                       // passes it)
   int ablate = 0;      // tersoff_set_ablation flags
   std::string tune_summary;  // last tersoff_autotune: choice and trial times
 

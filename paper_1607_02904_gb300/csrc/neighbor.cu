@@ -867,7 +867,7 @@ int launch_neighbor_build(Ctx* c, const double* x, cudaStream_t s) {
       bp.qref = c->d_qref;
       bp.pos64 = c->d_pos64;
       bp.fix64 = G.fix64;
-      bp.box = make_box64(G.L, G.fix64);
+      bp.box = c->box64;
       bp.kmask = c->d_kmask;
       TGB_CUDA(c, launch_pdl(c->precision == TERSOFF_FP64 ? k_bin_pack<true> : k_bin_pack<false>, nb, B, 0, s, n, x, g, bp, c->d_cell_of, c->d_cell_count,
                              c->d_qorg, c->d_flags));

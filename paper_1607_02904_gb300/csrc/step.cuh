@@ -245,7 +245,7 @@ inline PackArgs make_pack(Ctx* c, bool track, bool build = false) {
   a.posq = c->d_posq;
   a.pos64 = c->d_pos64;
   a.fix64 = c->grid.fix64;
-  a.box = make_box64(c->grid.L, c->grid.fix64);
+  a.box = c->box64;
   a.sys = c->n_sys > 0 ? c->d_sys : nullptr;
   a.atom_sys = c->d_atom_sys;
   a.flags = c->d_flags;

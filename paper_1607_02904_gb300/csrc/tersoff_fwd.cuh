@@ -233,7 +233,7 @@ template <class T> void set_pos64(const Ctx* c, FwdArgs<T>& a) {
   a.pos64 = c->d_pos64;
   a.fix64 = c->grid.fix64;
   a.long64 = c->grid.long64;
-  a.box = make_box64(c->grid.L, c->grid.fix64);
+  a.box = c->box64;
   // differences of up to four list radii fit the filter's 32 bits
   int keep = 30 - (int)ceil(log2(4.0 * c->r_list));
   if (keep > c->grid.fix64) keep = c->grid.fix64;
