@@ -156,8 +156,8 @@ int tersoff_neighbor_export(tersoff_ctx* ctx, int* cnt, int* nbr, int cap, void*
  * atom i (positive = repulsive); any output may be NULL. Outputs are
  * overwritten, not accumulated. On the FP64 path (tables inside its integer
  * formats, as all published ones are) a position that is not finite, or two
- * atoms at one place, make energy, virial and the forces of the atoms that
- * have them in their lists NaN. */
+ * atoms at one place, make energy, virial, the forces of the atoms that have
+ * them in their lists and those on these atoms' neighbours NaN. */
 int tersoff_compute(tersoff_ctx* ctx, const double* x, int n, double* energy,
                     double* forces, double* virial, void* stream);
 

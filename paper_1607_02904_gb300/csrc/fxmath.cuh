@@ -16,9 +16,9 @@
 // approximation by one step of second order. Every function's relative error
 // is below 2^-56 before its one rounding to double (the fixed-point logarithm's
 // absolute error below 2^-55); the reciprocal and the square root of doubles are
-// rounded correctly, as the operations that they stand for. Arguments outside a function's range (zero, subnormal,
-// infinite, NaN, or too large for the fixed-point formats) take the CUDA
-// functions or the FP64 formulas.
+// rounded correctly, as the operations that they stand for. Arguments outside a
+// function's range (zero, subnormal, infinite, NaN, or too large for the
+// fixed-point formats) take the CUDA functions or the FP64 formulas.
 //
 // Measured on GB300 against the CUDA functions: ten FP64 MD steps of 512,000 Si
 // atoms 11.1 -> 5.7 ms, one evaluation of 4,096 atoms 65 -> 52 us, a fitting

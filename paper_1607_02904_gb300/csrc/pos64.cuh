@@ -63,9 +63,9 @@ __device__ __forceinline__ long long nearest(long long d, long long L) {
   return d;
 }
 // the same on an axis of Lc units (out of line: inside the FP64 adjoint it cost 26
-// registers): the coarse words hi and hj (at bit s) tell the
-// image and whether the atoms are far apart (beyond any cutoff, which is below 4
-// units); the difference modulo 2^64 is the rest
+// registers): the coarse words hi and hj (at bit s) tell the image and whether the
+// atoms are far apart (beyond any cutoff, which is below 4 units); the difference
+// modulo 2^64 is the rest
 static __device__ __noinline__ long long nearest_long(long long d, long long L, int Lc, int hi, int hj, int s) {
   if (Lc < LONG64_EDGE) return nearest(d, L);
   int dc = ((hj >> s) & 1023) - ((hi >> s) & 1023);

@@ -508,10 +508,18 @@ __global__ void __launch_bounds__(LBLOCK, lanes_blocks<NS, MODE, BATCH, EV>()) k
           int jj, tj;
           odd |= Bond<double>::fixed(a, sh, pg, list[(size_t)s * a.n + ig], dx, dy, dz, jj, tj) || (dx | dy | dz) == 0;
         }
-        if (odd) {
+        if (odd) {  // as in lanes_atom, the forces on its neighbours too
           eg = fx::nan64();
           for (int p = 0; p < 6; ++p) w[p] = eg;
-          if (v.slots && in_short)
+          const bool st = v.slots && in_short;
+          for (int s = 0; s < c; ++s) {
+            const int jj = entry_atom(a, list, s, ig);
+            if (st)
+              store_slot<double>(a, a.contrib, recv_slot(a, s, ig, jj), eg, eg, eg);
+            else
+              atomic_add3(a.f, jj, eg, eg, eg);
+          }
+          if (st)
             store_slot<double>(a, a.own, (size_t)ig, eg, eg, eg);
           else
             atomic_add3(a.f, ig, eg, eg, eg);

@@ -120,3 +120,27 @@ def test_batches_show_them_in_their_system_only(T):
     assert torch.isnan(e[0]) and torch.isnan(f[7]).all()
     assert abs(e[1] - e0[1]) <= 1e-13 * abs(e0[1])
     assert (f[120:] - f0[120:]).abs().max() <= 1e-12 * f0[120:].abs().max()
+
+
+@pytest.mark.parametrize("scatter", [0, 1], ids=["gather", "atomic"])
+@pytest.mark.parametrize("case", list(systems()), ids=lambda c: c[0])
+def test_finite_forces_are_those_without_the_bad_position(T, case, scatter):
+    # no atom is pushed by a term that has the bad position in it: its force is NaN or
+    # what it is with all positions good (sums of the same terms: 1e-13 of the largest)
+    _, x, t, box, table = case
+    ctx = T.Context(T.FP64)
+    ctx.set_scatter(scatter)
+    ctx.params(table)
+    xd = torch.tensor(x, device="cuda")
+    ctx.neighbor_build(xd, torch.tensor(t, dtype=torch.int32, device="cuda"), box, min(4.0, 0.5 * box.min()))
+    f0, f = torch.zeros_like(xd), torch.zeros_like(xd)
+    ctx.compute(xd, None, f0, None)
+    for at, axis, value in ((5, 0, np.nan), (17, 1, np.inf), (40, 2, -np.inf)):
+        y = x.copy()
+        y[at, axis] = value
+        ctx.compute(torch.tensor(y, device="cuda"), None, f, None)
+        good = torch.isfinite(f).all(1)
+        assert not good[at]
+        if good.any():
+            assert (f[good] - f0[good]).abs().max() <= 1e-13 * f0.abs().max()
+    ctx.close()
