@@ -212,7 +212,7 @@ __device__ __forceinline__ Bo<T> bond_ad(T zeta, T be, T n) {
 // the warp totals go to the block and global sums in double. So the float
 // rounding of a gradient is that of its atoms' own terms, and which atoms meet
 // in a warp (their order comes from atomics) changes nothing above double
-// rounding; a plain float tree moved the gradient by 1e-9 to 1e-7 of its norm
+// rounding; a plain float tree moved the gradient by 1e-9 to 6e-7 of its norm
 // from one list build to the next. The FP64 pipe stays out of the loops.
 // NS == 1: one record. NS == 2 (mixed path): the 4 records (ti, *, *) of the
 // thread's centre species, summed once per centre species. Otherwise:
@@ -266,7 +266,8 @@ __device__ __forceinline__ void warp_sums(Get get, Out out) {
     e[0] = __fadd_rn(e[0], re);
     two_sum_acc(s[0], e[0], rs);
   }
-  if ((lane & (32 / C - 1)) == 0) out(mine, to_f64(s[0]) + to_f64(e[0]));
+  // (of an infinite sum the errors are NaN)
+  if ((lane & (32 / C - 1)) == 0) out(mine, to_f64(s[0]) + (fabsf(e[0]) < INFINITY ? to_f64(e[0]) : 0.0));
 }
 
 template <int NS, class T> struct Acc;

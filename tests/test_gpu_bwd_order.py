@@ -74,3 +74,25 @@ def test_fresh_batches_agree(T):
         got.append(torch.autograd.grad(loss, [tb])[0].numpy())
     for g in got[1:]:
         assert np.linalg.norm(g - got[0]) <= 1e-12 * np.linalg.norm(got[0])
+
+
+@pytest.mark.parametrize("names", [["Si"], ["Si", "C"]], ids=["si", "sic"])
+def test_infinite_sums_stay_infinite(T, names):
+    # an infinite energy weight: the A entries' terms are all +inf, the B entries' -inf
+    x, t, box = crystal((3, 3, 3), names, 0.05)
+    table = S.table_for(names, oracle.mix_tersoff89)
+    ctx = T.Context(T.MIXED)
+    ctx.params(table)
+    xd = torch.tensor(x, device="cuda")
+    ctx.neighbor_build(xd, torch.tensor(t, dtype=torch.int32, device="cuda"), box, 4.0)
+    g = torch.zeros(table.size, dtype=torch.float64, device="cuda")
+    ctx.backward(xd, torch.tensor([np.inf], dtype=torch.float64, device="cuda"), None, None, g)
+    g = g.cpu().numpy().reshape(-1, 14)
+    ctx.close()
+    ns = len(names)
+    for a in range(ns):
+        for b in range(ns):
+            if ns == 2 and a == b:
+                continue  # (no bonds between like atoms in zincblende)
+            r = g[(a * ns + b) * ns + b]
+            assert r[13] == np.inf and r[9] == -np.inf
